@@ -83,7 +83,7 @@ def parse():
     ap.add_argument("--n", type=int, default=0, help="override the particle count")
     ap.add_argument("--scenes", type=int, default=0, help="batched workload: override the bed count")
     ap.add_argument("--pgs-sync", type=int, default=-1, choices=[-1, 0, 1],
-                    help="solver sync between colours: 1 neighbour, 0 grid barrier (-1: library default)")
+                    help="solver sync between colours: 1 per particle, 0 grid barrier (-1: library default)")
     ap.add_argument("--pgs-blocks", type=int, default=0, help="solver CTAs (0: library default)")
     ap.add_argument("--pgs-shape", default="", help="solver CTA shape THREADSxPER_THREAD (e.g. 416x1)")
     ap.add_argument("--no-autotune", action="store_true",

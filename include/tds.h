@@ -435,20 +435,19 @@ tds_status tds_load_state(tds_scene *s, const void *buf, uint64_t bytes);
 /* ---- launch shapes ------------------------------------------------------------
  * Knobs of the GPU schedule (the paper, a CPU method, has none). Results do
  * not depend on them: every setting gives the same impulses and states bit
- * for bit. pgs_blocks: persistent solver CTAs (one per SM at most);
- * pgs_sync: between colours the solver either synchronises each CTA only
- * with the CTAs whose particles it can touch (1, the default) or all CTAs
- * with a grid barrier (0); colour_blocks: persistent colouring CTAs;
- * pgs_threads x pgs_per_thread: the solver CTA's threads and contacts per
- * thread, one of the compiled shapes 416x1 (the default, two CTAs per SM),
- * 768x1, 512x2, 640x2, 512x3 (one CTA per SM) and 256x1 (three CTAs per SM);
- * in each, the last warp stages the contact rows and the other threads solve
- * (both 0 keep the current shape).
+ * for bit. pgs_blocks: persistent solver CTAs (the co-resident ones at most);
+ * pgs_sync: between colours a contact waits only for the latest update of
+ * its own two particles (1, the default) or all CTAs meet at a grid barrier
+ * (0); colour_blocks: persistent colouring CTAs;
+ * pgs_threads x pgs_per_thread: the solver CTA's threads and the tiles of 32
+ * contact rows each of its warps keeps in flight, one of the compiled shapes
+ * 512x2 (the default), 768x1, 640x2, 512x3 (one CTA per SM), 416x1 (two CTAs
+ * per SM) and 256x1 (three CTAs per SM) (both 0 keep the current shape).
  * max_pgs_blocks / max_colour_blocks (read only) are the co-resident limits
  * (max_pgs_blocks for the current solver shape; a shape change with
  * pgs_blocks 0 lowers the solver CTAs to the new shape's limit if needed).
  * wait_limit_us: how long [microseconds] any CTA of the step's persistent
- * kernels waits for other CTAs (a grid barrier, a neighbour's progress flag)
+ * kernels waits for other CTAs (a grid barrier, a particle's record)
  * before it gives up: it latches TDS_ERR_BARRIER_TIMEOUT, every
  * CTA returns, and the next waiting call reports the error and rolls the
  * scene back (see the conventions above). Default 2 000 000 (2 s); a

@@ -3,7 +3,7 @@ own step).
 
 The knobs are the runtime launch shapes of ``tds_set_launch_config``: the
 persistent solver's CTA count and its synchronisation between colours
-(neighbour flags or a grid barrier) and the persistent colouring's CTA count.
+(per particle or a grid barrier) and the persistent colouring's CTA count.
 Every setting gives bit-identical results, so the tuner only picks the
 fastest: it times a few steps of the caller's own scene (continuing its
 motion) per candidate with CUDA events on the scene's stream and keeps the
@@ -64,9 +64,9 @@ def store_cache(key: str, entry: dict, path: str | None = None) -> None:
     os.replace(tmp, path)
 
 
-SYNC_MODES = (1, 0)  # neighbour synchronisation, grid barrier
-# solver CTA shapes the library compiles: (threads, contacts per thread, CTAs per SM)
-SHAPES = ((416, 1, 2), (768, 1, 1), (512, 2, 1), (640, 2, 1), (512, 3, 1), (256, 1, 3))
+SYNC_MODES = (1, 0)  # per particle, grid barrier
+# solver CTA shapes the library compiles: (threads, row tiles in flight per warp, CTAs per SM)
+SHAPES = ((512, 2, 1), (416, 1, 2), (768, 1, 1), (640, 2, 1), (512, 3, 1), (256, 1, 3))
 KEYS = ("pgs_blocks", "pgs_sync", "colour_blocks", "pgs_threads", "pgs_per_thread")
 
 

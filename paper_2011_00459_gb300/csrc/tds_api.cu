@@ -28,7 +28,8 @@ cudaError_t tds_mlp_loss_grad_launch(const void *packed, const float *X, const f
                                      float *grad, float *loss, cudaStream_t st);
 void tds_mlp_adam_launch(float *params, float *grad, float *mom, float *vel, uint32_t step, float lr,
                          cudaStream_t st);
-int tds_launch_predict(const DevPtrs &d, const StepConsts &k, cudaStream_t st);
+int tds_launch_predict(const DevPtrs &d, const StepConsts &k, int records, cudaStream_t st);
+int tds_launch_records(const DevPtrs &d, uint32_t n, cudaStream_t st);
 cudaError_t tds_launch_pgs(const DevPtrs &d, const StepConsts &k, uint32_t max_iters, float tol,
                            uint32_t every, int apply_warm, int blocks, int sync, int shape, cudaStream_t st);
 int tds_pgs_shapes();
@@ -174,7 +175,7 @@ struct tds_scene {
   std::vector<BoxF> host_boxes;
   bool geo_dirty = true;
   int pgs_blocks = 1, colour_blocks = 1;
-  int pgs_sync = 1;       // solver: 1 neighbour synchronisation, 0 grid barrier
+  int pgs_sync = 1;       // solver: 1 waits per particle, 0 grid barrier between colours
   int pgs_shape = 0;      // solver CTA shape (index of the compiled shapes)
   bool any_cutter = false;
   int max_pgs_blocks = 1, max_colour_blocks = 1;
@@ -375,6 +376,7 @@ Layout plan(const tds_scene_desc *descs, uint32_t S) {
 size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
   const uint32_t n = L.n, cap = L.cap;
   d.pos = c.take<float4>(n); d.pv = c.take<float4>(2 * (size_t)n);
+  d.rec = c.take<float4>(2 * (size_t)n);
   d.pid = c.take<uint32_t>(n); d.sid = c.take<uint32_t>(n);
   d.pos2 = c.take<float4>(n); d.pv2 = c.take<float4>(2 * (size_t)n);
   d.pid2 = c.take<uint32_t>(n); d.sid2 = c.take<uint32_t>(n);
@@ -395,6 +397,7 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
   d.inc_cursor = c.take<uint32_t>(n); d.inc_ent = c.take<uint2>(2 * (size_t)cap);
   d.prio = c.take<unsigned long long>(cap);
   d.colour = c.take<uint8_t>(cap);
+  d.cmask = c.take<ulonglong2>(n);
   d.wait = c.take<int32_t>(cap);
   d.frontier0 = c.take<uint32_t>(cap); d.frontier1 = c.take<uint32_t>(cap);
   d.ntiles = L.ntiles;
@@ -408,6 +411,8 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
   d.p_ab = c.take<uint2>(pc);
   d.p_rn = c.take<float4>(pc); d.p_rq = c.take<float4>(pc);
   d.p_rm = c.take<float2>(pc);
+  d.p_im = c.take<float4>(pc);
+  d.p_rk = c.take<uint32_t>(pc);
   d.p_sv = c.take<float4>(pc); d.p_sw = c.take<float4>(pc);
   d.p_la = c.take<float4>(pc); d.p_lb = c.take<float2>(pc);
   d.p_il = c.take<float4>(pc); d.p_il2 = c.take<float4>(pc);
@@ -436,8 +441,7 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
   d.scene_res = c.take<float>(L.S);
   d.scene_iters = c.take<uint32_t>(L.S);
   d.bar = c.take<uint32_t>(2);
-  d.prog = c.take<uint32_t>(kProgStride * (size_t)pgs_blocks);
-  d.rng = c.take<uint32_t>(2 * (size_t)pgs_blocks);
+  d.tiles = c.take<uint2>((size_t)cap / 32 + TDS_NBUCKETS);
   size_t m = L.ncells + 1;
   if (m < n) m = n;
   if (m < (size_t)TDS_NBUCKETS * L.ntiles) m = (size_t)TDS_NBUCKETS * L.ntiles;
@@ -473,7 +477,7 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
 }
 
 int pgs_blocks_for(uint32_t n, int max_coop) {
-  int b = (int)((n + 511) / 512);
+  int b = (int)((n + 127) / 128);
   if (b < 1) b = 1;
   return b < max_coop ? b : max_coop;
 }
@@ -839,7 +843,7 @@ tds_status enqueue_step(tds_scene *s, cudaEvent_t *E, uint64_t &launches, bool c
   // the learned warm start also reads the previous step's impulses
   int use_prev = (D.warm_start != TDS_WARM_COLD) && s->have_prev;
   launches += tds_launch_narrowphase(d, s->k, use_prev, s->st);
-  launches += tds_launch_predict(d, s->k, s->st);
+  launches += tds_launch_predict(d, s->k, D.impact_iters == 0, s->st);
   if (E) CUDA_TRY(cudaEventRecordWithFlags(E[2], s->st, evf));
   launches += tds_launch_colouring(d, s->L.n, s->L.cap, s->colour_blocks, 256, s->st);
   d.targ = s->recording ? s->x.targ : nullptr;
@@ -854,7 +858,7 @@ tds_status enqueue_step(tds_scene *s, cudaEvent_t *E, uint64_t &launches, bool c
   launches += tds_launch_bucketing(d, s->L.cap, s->st);
   if (D.impact_iters > 0) {
     CUDA_TRY(tds_launch_impact(d, s->k, D.restitution, D.impact_speed, D.impact_iters, s->pgs_blocks, s->st));
-    launches += 1;
+    launches += 1 + tds_launch_records(d, s->L.n, s->st);
   }
   if (E) CUDA_TRY(cudaEventRecordWithFlags(E[3], s->st, evf));
   CUDA_TRY(tds_launch_pgs(d, s->k, D.max_iters, D.tol, D.residual_every, use_prev || learned, s->pgs_blocks,

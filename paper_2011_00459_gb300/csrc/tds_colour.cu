@@ -194,6 +194,38 @@ __global__ void k_colour_rounds(DevPtrs d) {
   if (blockIdx.x == 0 && threadIdx.x == 0) d.ctr[CTR_ROUNDS] = round + 1;
 }
 
+// The colours of every particle's contacts as bits (a contact left without a
+// colour, only after a latched error, counts as the last one).
+__global__ void k_colour_masks(DevPtrs d, uint32_t n) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const uint32_t s = d.inc_start[i], e = d.inc_start[i + 1];
+    unsigned long long lo = 0ull, hi = 0ull;
+    for (uint32_t m0 = s; m0 < e; m0 += kBatch) {
+      uint32_t col[kBatch];
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) col[q] = m0 + q < e ? (uint32_t)d.colour[d.inc_ent[m0 + q].x] : 0x100u;
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        if (col[q] == 0x100u) continue;
+        const uint32_t b = min(col[q], (uint32_t)TDS_MAX_COLOURS - 1u);
+        if (b < 64u) lo |= 1ull << b;
+        else hi |= 1ull << (b - 64u);
+      }
+    }
+    d.cmask[i] = make_ulonglong2(lo, hi);
+  }
+}
+
+// Of a contact of colour col at a particle with these colours: how many of the
+// particle's contacts come before it in a sweep (its rank), and how many there
+// are (the degree).
+__device__ __forceinline__ uint32_t rank_degree(ulonglong2 m, uint32_t col) {
+  const uint32_t nlo = __popcll(m.x), nhi = __popcll(m.y);
+  const uint32_t rank = col < 64u ? __popcll(m.x & ((1ull << col) - 1ull))
+                                  : nlo + __popcll(m.y & ((1ull << (col - 64u)) - 1ull));
+  return rank | ((nlo + nhi) << 8);
+}
+
 // ---- stable counting sort of contacts by bucket = 2 colour + static? ------
 // Colours are < TDS_MAX_COLOURS once the colouring finished; a contact left
 // uncoloured (only after a latched error) is clamped into the last bucket.
@@ -269,15 +301,25 @@ __global__ void __launch_bounds__(256) k_bucket_scatter(DevPtrs d) {
     __syncthreads();
     if (live) {
       uint32_t p = wcnt[warp][bk] + rank_in_warp + d.bpad[bk];
+      const uint2 ab = d.c_ab[c];
       d.order[p] = c;
-      d.p_ab[p] = d.c_ab[c];
+      d.p_ab[p] = ab;
+      uint32_t rk = rank_degree(d.cmask[ab.x], bk >> 1);
+      float4 im = make_float4(d.pv[2 * (size_t)ab.x].w, d.pv[2 * (size_t)ab.x + 1].w, 0.f, 0.f);
+      if (is_dyn(ab.y)) {
+        rk |= rank_degree(d.cmask[ab.y], bk >> 1) << 16;
+        im.z = d.pv[2 * (size_t)ab.y].w;
+        im.w = d.pv[2 * (size_t)ab.y + 1].w;
+      }
+      d.p_im[p] = im;
+      d.p_rk[p] = rk;
       d.p_rn[p] = d.c_rn[c];
       d.p_rq[p] = d.c_rq[c];
       d.p_rm[p] = d.c_rm[c];
       if (bk & 1u) { d.p_sv[p] = d.c_sv[c]; d.p_sw[p] = d.c_sw[c]; }
       d.p_la[p] = d.c_la[c];
       d.p_lb[p] = d.c_lb[c];
-      if (d.nscenes > 1) atomicAdd(d.scq_cnt + (size_t)d.sid[d.c_ab[c].x] * TDS_NBUCKETS + bk, 1u);
+      if (d.nscenes > 1) atomicAdd(d.scq_cnt + (size_t)d.sid[ab.x] * TDS_NBUCKETS + bk, 1u);
     }
     __syncthreads();
   }
@@ -354,7 +396,8 @@ int tds_launch_colouring(const DevPtrs &d, uint32_t n, uint32_t cap, int coop_bl
   void *args[] = {&dd};
   cudaLaunchCooperativeKernel((const void *)k_colour_rounds, dim3(coop_blocks), dim3(coop_threads),
                               args, 0, st);
-  return 8;
+  k_colour_masks<<<(n + 255) / 256 < 152 * 16 ? (n + 255) / 256 : 152 * 16, 256, 0, st>>>(d, n);
+  return 9;
 }
 
 // Contact rows (and initial impulses) into the padded colour order.

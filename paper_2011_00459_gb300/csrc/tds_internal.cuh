@@ -32,8 +32,6 @@ struct BoxF {
 // Geometry and material of one scene of a batch (device table; a single
 // scene is a batch of one). Scenes never touch: each has its own block of
 // broadphase cells, so its particles keep their own coordinates.
-constexpr uint32_t kProgStride = 32;  // words between the solver's progress flags
-
 struct SceneGeo {
   float lo[3];                 // origin of the scene's broadphase cells
   int hf_nx, hf_ny;            // heightfield (hf_nx == 0: none)
@@ -100,6 +98,7 @@ struct DevPtrs {
   // particles, slot order (re-sorted by cell every step)
   float4 *pos;                // (x, y, z, r)
   float4 *pv;                 // 32-byte state record per particle: [2i] (v, 1/m), [2i+1] (w, 1/I)
+  float4 *rec;                // solver: versioned velocity record per particle (see tds_solve.cu)
   uint32_t *pid;
   uint32_t *sid;              // scene of the particle
   float4 *pos2, *pv2;         // reorder targets
@@ -120,6 +119,7 @@ struct DevPtrs {
   uint2 *inc_ent;             // (contact id, high word of its priority) per incidence
   unsigned long long *prio;   // colouring priority per contact
   uint8_t *colour;
+  ulonglong2 *cmask;          // per slot: the colours of its contacts, a bit each
   int32_t *wait;
   uint32_t *frontier0, *frontier1;
   // bucketing into colour order
@@ -130,6 +130,8 @@ struct DevPtrs {
   uint2 *p_ab;
   float4 *p_rn, *p_rq;
   float2 *p_rm;
+  float4 *p_im;               // 1/m_a, 1/I_a, 1/m_b, 1/I_b (0 for a static side)
+  uint32_t *p_rk;             // rank and degree of the contact at a, then at b (a byte each)
   float4 *p_sv, *p_sw;
   float4 *p_la;
   float2 *p_lb;
@@ -138,7 +140,7 @@ struct DevPtrs {
   float4 *prev_l0[2], *prev_l1[2];
   // scalars and scratch
   uint32_t recolour;          // colour every contact every recolour-th step (1: every step)
-  unsigned long long wait_ns; // limit of every wait on other CTAs (grid barriers, neighbour flags)
+  unsigned long long wait_ns; // limit of every wait on other CTAs (grid barriers, particle records)
                               // before the wait gives up and latches DEV_ERR_BARRIER
   int32_t *err;
   uint32_t *ctr;              // see CTR_* below
@@ -156,9 +158,7 @@ struct DevPtrs {
   float *scene_res;           // per scene: residual at its last check of the last step
   uint32_t *scene_iters;      // per scene: sweeps of the last step
   uint32_t *bar;              // grid barrier: [0] arrivals, [1] generation
-  uint32_t *prog;             // solver neighbour sync: last colour phase published per CTA,
-                              // one flag per kProgStride words (own 128-byte line)
-  uint32_t *rng;              // solver neighbour sync: touched slot range [lo, hi] per CTA
+  uint2 *tiles;               // solver: the warps' row tiles (first contact, contacts | bucket << 8)
   uint32_t *scan_tmp;
   float *stage;               // 9 n floats for reads
   float *tool_out;            // 6 floats per scene

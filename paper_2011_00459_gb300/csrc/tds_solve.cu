@@ -6,32 +6,21 @@
 // colour: within a colour no two contacts share a particle, so all of them
 // are updated in parallel and the result equals sequential Gauss-Seidel in
 // colour-major order. One persistent, co-resident kernel runs the whole
-// solve, each CTA waiting between colours only for the CTAs whose particles
-// overlap its own (or, as an option, at a grid barrier): first
-// v = M^-1 (p + G^T lambda_0) from the warm-start impulses, then the sweeps,
-// with residual checks where the tolerance asks for them. Per contact and
+// solve, each contact waiting only for the versions of its two particles
+// that the order gives it (or, as an option, every colour at a grid barrier):
+// first v = M^-1 (p + G^T lambda_0) from the warm-start impulses, then the
+// sweeps, with residual checks where the tolerance asks for them. Per contact and
 // sweep: the normal row (clamped at -f_c), the 2-D tangent rows projected on
 // the Coulomb disk mu |Lambda_n|, the 3 rolling rows projected on the ball
 // rbar mu_r |Lambda_n| (Eqs. signCoul1-3), each followed by
 // v += M^-1 G^T dLambda. Particle velocities are read and written through L2
-// (ld.global.cg / st.global.cg) because other SMs update them between colours.
+// because other SMs update them between colours.
 #include "tds_internal.cuh"
 
 namespace {
 
 __device__ __forceinline__ bool is_dyn(uint32_t b) { return (b & TDS_STATIC) == 0u; }
 
-__global__ void k_predict(DevPtrs d, StepConsts k) {
-  if (step_failed(d)) return;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < k.n; i += gridDim.x * blockDim.x) {
-    float4 v = d.pv[2 * i];
-    if (v.w == 0.0f) continue;  // dormant reserve slot (1/m = 0): no gravity
-    v.x += k.dt * k.g[0];
-    v.y += k.dt * k.g[1];
-    v.z += k.dt * k.g[2];
-    d.pv[2 * i] = v;
-  }
-}
 
 struct Side {
   float3 v, w;
@@ -131,30 +120,39 @@ __device__ __forceinline__ float diag_r(const Side &A, const Side &B, float sig_
   return __fadd_rn(__fadd_rn(A.iI, B.iI), sig_r);
 }
 
+// What an update of a contact needs besides the velocities: the inverse
+// diagonals and the tangent basis.
+struct Pre {
+  float iDn, iDt, iDr;
+  float3 t1, t2;
+};
+__device__ __forceinline__ Pre prepare_update(const Row &r, const Side &A, const Side &B, float sig_t, float sig_r) {
+  Pre q;
+  q.iDn = __frcp_rn(diag_n(r, A, B));
+  q.iDt = __frcp_rn(diag_t(r, A, B, sig_t));
+  q.iDr = __frcp_rn(diag_r(A, B, sig_r));
+  onb(r.n, q.t1, q.t2);
+  return q;
+}
 // One projected Gauss-Seidel update of one contact.
-__device__ __forceinline__ void pgs_update(const Row &r, Side &A, Side &B, float4 &L0, float2 &L1,
+__device__ __forceinline__ void pgs_update(const Row &r, const Pre &q, Side &A, Side &B, float4 &L0, float2 &L1,
                                            float sig_t, float sig_r) {
   // normal row
-  const float iDn = __frcp_rn(diag_n(r, A, B));
   const float res = __fsub_rn(__fmaf_rn(r.Sn, L0.x, dot(r.n, B.v - A.v)), r.qn);
-  const float ln = fmaxf(__fmaf_rn(-res, iDn, L0.x), -r.fc);
+  const float ln = fmaxf(__fmaf_rn(-res, q.iDn, L0.x), -r.fc);
   apply_normal(r, A, B, __fsub_rn(ln, L0.x));
   L0.x = ln;
   // tangent rows (Coulomb disk)
-  float3 t1, t2;
-  onb(r.n, t1, t2);
-  const float iDt = __frcp_rn(diag_t(r, A, B, sig_t));
   const float3 u = slip(r, A, B);
-  float y1 = __fmaf_rn(-__fmaf_rn(sig_t, L0.y, dot(t1, u)), iDt, L0.y);
-  float y2 = __fmaf_rn(-__fmaf_rn(sig_t, L0.z, dot(t2, u)), iDt, L0.z);
+  float y1 = __fmaf_rn(-__fmaf_rn(sig_t, L0.y, dot(q.t1, u)), q.iDt, L0.y);
+  float y2 = __fmaf_rn(-__fmaf_rn(sig_t, L0.z, dot(q.t2, u)), q.iDt, L0.z);
   disk(y1, y2, __fmul_rn(r.mu, fabsf(ln)));
-  apply_tangent(r, A, B, axpy(__fsub_rn(y2, L0.z), t2, __fsub_rn(y1, L0.y) * t1));
+  apply_tangent(r, A, B, axpy(__fsub_rn(y2, L0.z), q.t2, __fsub_rn(y1, L0.y) * q.t1));
   L0.y = y1;
   L0.z = y2;
   // rolling rows (ball)
-  const float iDr = __frcp_rn(diag_r(A, B, sig_r));
   const float3 lr = make_float3(L0.w, L1.x, L1.y);
-  float3 y = axpy(-iDr, axpy(sig_r, lr, B.w - A.w), lr);
+  float3 y = axpy(-q.iDr, axpy(sig_r, lr, B.w - A.w), lr);
   ball(y, __fmul_rn(r.rmu, fabsf(ln)));
   apply_rolling(A, B, y - lr);
   L0.w = y.x;
@@ -226,467 +224,407 @@ struct SolveArgs {
   uint32_t max_iters, every;
   float tol, sig_t, sig_r;
   int apply_warm;
-  int sync;  // between colours: 0 grid barrier, 1 neighbour synchronisation
+  int sync;  // between colours: 0 grid barrier, 1 the particle records' versions alone
   uint32_t n;  // particle slots
 };
 
 // ---------------------------------------------------------------------------
-// Staging of the contact rows and impulses with bulk copies (TMA)
+// The solver's order without barriers: versioned particle records
 // ---------------------------------------------------------------------------
-// CTA shapes compiled: (threads, contacts per thread, co-resident CTAs per
-// SM the register budget is sized for); launch configurations choose one by
-// index. In every shape the last warp stages the waves and the others solve
-// (a wave is (threads - 32) x contacts per thread, see pgs_wave). The first
-// is the default, measured fastest on the 1M bed: two 416-thread CTAs per SM
-// (384 solving threads each, one contact per thread). Each colour phase is a
-// latency chain of which a thread's serial updates are a large part, and the
-// second CTA keeps the SM busy while the first waits.
-constexpr int kShapes[][3] = {{416, 1, 2}, {768, 1, 1}, {512, 2, 1}, {640, 2, 1}, {512, 3, 1}, {256, 1, 3}};
+// Within a sweep a particle's contacts update it in colour order, one at a
+// time. The contact with the k-th smallest colour among the particle's deg
+// contacts (its rank) therefore reads the record that the update before it
+// wrote: in pass p (pass 0: the warm start, if there is one, then the sweeps)
+// exactly the version p deg + k, counting every update from 0. The record
+// carries its version, so a contact waits for its two particles only, by
+// reading their records until they hold the versions it needs, and hands
+// them on by storing version + 1 with the new velocities. A version has one
+// reader and one writer, so nothing is ever overwritten before it is read.
+// All warps are co-resident and take their contacts in (pass, colour) order;
+// the earliest outstanding contact needs only finished ones, so some warp
+// always advances.
+//
+// A record is one 32-byte sector, moved by one 256-bit access: (v, version),
+// (w, check). The memory model promises single 32-bit words only; check is
+// the exclusive or of the other seven, so a mixture of two versions does not
+// pass for either.
+constexpr uint32_t kCheckSeed = 0x5bd1e995u;
+
+__device__ __forceinline__ float check_word(float4 v, float3 w) {
+  return __uint_as_float(__float_as_uint(v.x) ^ __float_as_uint(v.y) ^ __float_as_uint(v.z) ^ __float_as_uint(v.w) ^
+                         __float_as_uint(w.x) ^ __float_as_uint(w.y) ^ __float_as_uint(w.z) ^ kCheckSeed);
+}
+__device__ __forceinline__ void ld_rec(const float4 *rec, float4 &v, float4 &w) {
+  asm volatile("ld.relaxed.gpu.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w), "=f"(w.x), "=f"(w.y), "=f"(w.z), "=f"(w.w)
+               : "l"(rec)
+               : "memory");
+}
+__device__ __forceinline__ void st_rec(float4 *rec, float3 v, float3 w, uint32_t version) {
+  const float4 a = make_float4(v.x, v.y, v.z, __uint_as_float(version));
+  asm volatile("st.relaxed.gpu.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(rec), "f"(a.x), "f"(a.y),
+               "f"(a.z), "f"(a.w), "f"(w.x), "f"(w.y), "f"(w.z), "f"(check_word(a, w))
+               : "memory");
+}
+__device__ __forceinline__ bool is_version(float4 v, float4 w, uint32_t version) {
+  return __float_as_uint(v.w) == version && __float_as_uint(w.w) == __float_as_uint(check_word(v, f3(w)));
+}
+
+// v* = v + h g, and (records != 0) the solver's records at version 0.
+__global__ void k_predict(DevPtrs d, StepConsts k, int records) {
+  if (step_failed(d)) return;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < k.n; i += gridDim.x * blockDim.x) {
+    float4 v = d.pv[2 * i];
+    if (v.w != 0.0f) {  // (1/m = 0: a dormant reserve slot, no gravity)
+      v.x += k.dt * k.g[0];
+      v.y += k.dt * k.g[1];
+      v.z += k.dt * k.g[2];
+      d.pv[2 * i] = v;
+    }
+    if (records) st_rec(d.rec + 2 * (size_t)i, f3(v), f3(d.pv[2 * i + 1]), 0u);
+  }
+}
+
+// The solver's records at version 0 from the particle state (after the impact
+// stage, which changes the predicted velocities).
+__global__ void k_records(DevPtrs d, uint32_t n) {
+  if (step_failed(d)) return;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    st_rec(d.rec + 2 * (size_t)i, f3(d.pv[2 * i]), f3(d.pv[2 * i + 1]), 0u);
+}
+
+// CTA shapes compiled: (threads, row tiles in flight per warp, co-resident
+// CTAs per SM the register budget is sized for); launch configurations choose
+// one by index, the first is the default.
+constexpr int kShapes[][3] = {{512, 2, 1}, {416, 1, 2}, {768, 1, 1}, {640, 2, 1}, {512, 3, 1}, {256, 1, 3}};
 constexpr int kNumShapes = 6;
-constexpr int kStages = 2;                           // waves in flight
+constexpr int kStages = 1;                           // ring stages per row tile in flight (and one in use)
 constexpr uint32_t kFirstCheck = 5;                  // first residual check in adaptive mode
 constexpr uint32_t kResSum = 256;                    // residual: threads adding up a large scene's chunks
 constexpr uint32_t kWarpChunks = 1024;               // residual: scenes with at most this many chunks
                                                      // are added by one warp, larger ones by the CTA
-// per contact: ab 8 | (n, la) 16 | (lb, q_n, Sigma_n, f_c) 16 | (mu, rbar mu_r) 8 |
-//              impulses (n, t1, t2, r.x) 16 | (r.y, r.z) 8
-constexpr size_t kRowBytes = 72;
-constexpr size_t kOffAb = 0, kOffRn = 8, kOffRq = 24, kOffRm = 40, kOffLa = 48, kOffLb = 64;  // x wave size
-__host__ __device__ constexpr size_t stage_bytes(int wave) { return (size_t)wave * kRowBytes; }
-__host__ __device__ constexpr size_t pgs_smem(int wave) { return kStages * stage_bytes(wave); }
-// The last warp of a CTA stages the waves (bulk copies take the issuing
-// thread a long time each: on a computing warp they would hold up every
-// wave's barrier); the other warps solve, one wave = their threads x the
-// contacts per thread.
-__host__ __device__ constexpr int pgs_wave(int threads, int per_thread) { return (threads - 32) * per_thread; }
+// A row tile: the rows and impulses of 32 contacts of one bucket (one lane
+// each), field by field. Per contact: (n, la) 16 | (lb, q_n, Sigma_n, f_c) 16 |
+// (1/m_a, 1/I_a, 1/m_b, 1/I_b) 16 | impulses (n, t1, t2, r.x) 16 | ab 8 |
+// (mu, rbar mu_r) 8 | impulses (r.y, r.z) 8 | ranks and degrees 4 | index 4
+constexpr size_t kRowBytes = 96;
+constexpr size_t kOffRn = 0, kOffRq = 16, kOffIm = 32, kOffLa = 48, kOffAb = 64, kOffRm = 72, kOffLb = 80, kOffRk = 88,
+                 kOffIx = 92;  // x 32 contacts
+constexpr size_t kTileBytes = 32 * kRowBytes;
+__host__ __device__ constexpr int ring_tiles(int per_thread) { return kStages * per_thread + 1; }
+__host__ __device__ constexpr size_t pgs_smem(int threads, int per_thread) {
+  return (size_t)(threads / 32) * ring_tiles(per_thread) * kTileBytes;
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
-__device__ __forceinline__ void mbar_init(unsigned long long *bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+template <int B>
+__device__ __forceinline__ void cp_async(uint32_t dst, const void *src) {
+  if (B == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(B) : "memory");
 }
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long *bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_test(unsigned long long *bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait of one thread for a phase of a stage barrier; false (error
-// latched) when it has waited longer than limit_ns, or (if early) at once
-// when the step has already failed. The wait for the copies still in flight
-// before a CTA exits is not early: it gives those copies their full time.
-__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, uint32_t parity, int32_t *err,
-                                          unsigned long long limit_ns, bool early = true) {
-  unsigned long long t0 = 0;
-  for (unsigned k = 0;; ++k) {
-    if (mbar_test(bar, parity)) return true;
-    if (k == 0) t0 = global_ns();
-    if ((k & 15u) == 15u) {
-      if (early && *(volatile int32_t *)err != 0) return false;  // the step has failed already
-      if (global_ns() - t0 > limit_ns) {
-        latch_error(err, DEV_ERR_BARRIER);
-        return false;
-      }
-    }
-  }
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// One lane copies its own contact's row; only that lane reads it, so its own
+// wait for the copy is all the synchronisation there is.
+__device__ __forceinline__ void stage_row(const DevPtrs &d, uint32_t p, uint32_t stage, uint32_t lane) {
+  cp_async<16>(stage + kOffRn * 32 + 16 * lane, d.p_rn + p);
+  cp_async<16>(stage + kOffRq * 32 + 16 * lane, d.p_rq + p);
+  cp_async<16>(stage + kOffIm * 32 + 16 * lane, d.p_im + p);
+  cp_async<16>(stage + kOffLa * 32 + 16 * lane, d.p_la + p);
+  cp_async<8>(stage + kOffAb * 32 + 8 * lane, d.p_ab + p);
+  cp_async<8>(stage + kOffRm * 32 + 8 * lane, d.p_rm + p);
+  cp_async<8>(stage + kOffLb * 32 + 8 * lane, d.p_lb + p);
+  cp_async<4>(stage + kOffRk * 32 + 4 * lane, d.p_rk + p);
 }
 
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes,
-                                         unsigned long long *bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-
-// Segments: colour c has two, 2c (its particle-pair bucket) and 2c + 1 (its
-// static bucket). Each CTA takes the same share [lo, hi) of both, starting at
-// a multiple of 4 contacts, so its work in every colour lies in the same
-// stretch of slot order (buckets keep the owner order).
-__device__ __forceinline__ void seg_chunk(const DevPtrs &d, uint32_t g, uint32_t &lo, uint32_t &hi) {
-  const uint32_t s = d.bstart[g], e = d.bend[g];
-  uint32_t q = (e - s + gridDim.x - 1) / gridDim.x;
-  q = (q + 3u) & ~3u;
-  lo = min(s + blockIdx.x * q, e);
-  hi = min(lo + q, e);
-}
-
-// One wave of a colour: up to W contacts of this CTA's pair chunk
-// [lo1, hi1), then of its static chunk [lo2, hi2). The pair part n1 sits at
-// stage entries [0, n1), the static part n2 at [n1e, n1e + n2) with n1e = n1
-// rounded up to even (8-byte fields are copied in 16-byte pairs); n1e + n2 <=
-// W. Waves of a colour: the pair chunk in W pieces, the last one
-// topped up with static contacts, then the rest of the static chunk.
-struct WaveDesc {
-  uint32_t a1, n1, n1e, a2, n2;
-};
-
-__device__ __forceinline__ uint32_t waves_of(uint32_t L1, uint32_t L2, uint32_t W) {
-  const uint32_t W1 = (L1 + W - 1) / W;
-  uint32_t first2 = 0;  // static contacts in the last pair wave
-  if (W1 > 0) {
-    const uint32_t n1 = L1 - (W1 - 1) * W;
-    first2 = min(L2, W - ((n1 + 1u) & ~1u));
-  }
-  return W1 + (L2 - first2 + W - 1) / W;
-}
-
-__device__ __forceinline__ WaveDesc wave_desc(uint32_t lo1, uint32_t hi1, uint32_t lo2, uint32_t hi2, uint32_t w,
-                                              uint32_t W) {
-  const uint32_t L1 = hi1 - lo1, L2 = hi2 - lo2;
-  const uint32_t W1 = (L1 + W - 1) / W;
-  WaveDesc q{0, 0, 0, lo2, 0};
-  uint32_t first2 = 0;
-  if (W1 > 0) {
-    const uint32_t n1 = L1 - (W1 - 1) * W;
-    first2 = min(L2, W - ((n1 + 1u) & ~1u));
-  }
-  if (w < W1) {
-    q.a1 = lo1 + w * W;
-    q.n1 = min(W, L1 - w * W);
-    q.n1e = (q.n1 + 1u) & ~1u;
-    if (w == W1 - 1) q.n2 = first2;
+// The row and both sides of contact p as the residual pass reads them (after
+// a grid barrier: no update is in flight).
+__device__ __forceinline__ Row settled_pair(const DevPtrs &d, uint32_t p, Side &A, Side &B) {
+  Row r = load_row(d, p);
+  const float4 im = d.p_im[p];
+  float4 v, w;
+  ld_rec(d.rec + 2 * (size_t)r.ab.x, v, w);
+  A = Side{f3(v), f3(w), im.x, im.y};
+  if (r.dyn) {
+    ld_rec(d.rec + 2 * (size_t)r.ab.y, v, w);
+    B = Side{f3(v), f3(w), im.z, im.w};
   } else {
-    const uint32_t done = first2 + (w - W1) * W;
-    q.a2 = lo2 + done;
-    q.n2 = min(W, L2 - done);
+    B = Side{r.sv, r.sw, 0.f, 0.f};
   }
-  return q;
+  return r;
 }
 
-// Walks the (sweep, colour, wave) sequence of this CTA's staged waves.
-struct WaveSeq {
-  uint32_t sweep, col, w;
-  __device__ bool valid(uint32_t max_iters) const { return sweep < max_iters; }
-  // moves to the next wave, skipping colours without waves for this CTA
-  __device__ void advance(const uint32_t *nw, uint32_t ncol, uint32_t max_iters) {
-    ++w;
-    while (sweep < max_iters && w >= nw[col]) {
-      w = 0;
-      if (++col >= ncol) { col = 0; ++sweep; }
-    }
-  }
-};
-
-__device__ __forceinline__ void stage_range(const DevPtrs &d, uint32_t p0, uint32_t cnt, uint32_t at,
-                                            unsigned char *stage, unsigned long long *bar, uint32_t W) {
-  const uint32_t cnt2 = (cnt + 1u) & ~1u;  // 8-byte fields copied in pairs (16-byte multiples)
-  bulk_g2s(stage + kOffAb * W + 8u * at, d.p_ab + p0, 8u * cnt2, bar);
-  bulk_g2s(stage + kOffRn * W + 16u * at, d.p_rn + p0, 16u * cnt, bar);
-  bulk_g2s(stage + kOffRq * W + 16u * at, d.p_rq + p0, 16u * cnt, bar);
-  bulk_g2s(stage + kOffRm * W + 8u * at, d.p_rm + p0, 8u * cnt2, bar);
-  bulk_g2s(stage + kOffLa * W + 16u * at, d.p_la + p0, 16u * cnt, bar);
-  bulk_g2s(stage + kOffLb * W + 8u * at, d.p_lb + p0, 8u * cnt2, bar);
-}
-
-__device__ __forceinline__ uint32_t range_bytes(uint32_t cnt) {
-  return cnt ? 3u * 16u * cnt + 3u * 8u * ((cnt + 1u) & ~1u) : 0u;
-}
-
-__device__ __forceinline__ void issue_wave(const DevPtrs &d, const WaveSeq &q, const uint32_t *lo,
-                                           const uint32_t *hi, unsigned char *stage,
-                                           unsigned long long *bar, uint32_t W) {
-  const WaveDesc w = wave_desc(lo[2 * q.col], hi[2 * q.col], lo[2 * q.col + 1], hi[2 * q.col + 1], q.w, W);
-  mbar_expect_tx(bar, range_bytes(w.n1) + range_bytes(w.n2));
-  if (w.n1) stage_range(d, w.a1, w.n1, 0, stage, bar, W);
-  if (w.n2) stage_range(d, w.a2, w.n2, w.n1e, stage, bar, W);
-}
-
-// Neighbour synchronisation. Every CTA touches particles only inside its slot
-// range [rng_lo, rng_hi] (both sides of all its contacts, all colours); its
-// neighbours are the CTAs whose ranges overlap it (a symmetric relation).
-// Before colour phase t a CTA waits until each neighbour has published phase
-// t - 1; after its own stores of phase t it publishes t. Every write to a
-// particle before phase t then comes from a neighbour that has finished it,
-// and no neighbour can still be reading a particle this CTA writes, so the
-// result equals the grid-barrier order bit for bit. The least advanced CTA
-// never waits, so the scheme cannot deadlock. The threads poll the
-// neighbours between them; waits are bounded like grid_barrier.
-__device__ __forceinline__ bool neighbour_wait(const DevPtrs &d, uint32_t jlo, uint32_t jhi, uint32_t target,
-                                               int *s_fail) {
-  // thread t polls neighbours jlo + t, jlo + t + blockDim.x, ... (a range can
-  // be wider than the CTA when few contacts of a colour spread over the bed)
-  for (uint32_t j = jlo + threadIdx.x; j <= jhi; j += blockDim.x) {
-    if (j == blockIdx.x) continue;
-    unsigned long long t0 = 0;
-    for (unsigned spins = 0;; ++spins) {
-      uint32_t cur;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cur) : "l"(d.prog + kProgStride * j) : "memory");
-      if ((int32_t)(cur - target) >= 0) break;
-      if ((spins & 31u) == 31u) {
-        if (*(volatile int32_t *)d.err != 0) { *s_fail = 1; break; }
-        unsigned long long t = global_ns();
-        if (t0 == 0) t0 = t;
-        else if (t - t0 > d.wait_ns) {
-          latch_error(d.err, DEV_ERR_BARRIER);
-          *s_fail = 1;
-          break;
-        }
-      }
-    }
-    if (*(volatile int *)s_fail) break;
-  }
-  __syncthreads();
-  return *s_fail == 0;
-}
-
-// Publishes phase t of this CTA; the caller has passed a __syncthreads after
-// the phase's stores (the release is cumulative over them).
-__device__ __forceinline__ void publish(const DevPtrs &d, uint32_t t) {
-  if (threadIdx.x == 0)
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(d.prog + kProgStride * blockIdx.x), "r"(t)
-                 : "memory");
-}
-
-// The persistent solver: kMinBlocks co-resident CTAs per SM; between colours
-// either a grid barrier or neighbour synchronisation. The rows and impulses
-// of each wave (up to kWave contacts of one segment) are staged in shared
-// memory by bulk copies that the CTA's last warp issues ahead, so they stream
-// from HBM while earlier colours are solved and synchronised; each solving
-// thread then gathers both sides of its kPerThread contacts (through L2)
-// before solving any of them (contacts of one colour touch disjoint
-// particles).
-template <int kPgsThreads, int kPerThread, int kMinBlocks>
-__global__ void __launch_bounds__(kPgsThreads, kMinBlocks) k_pgs(DevPtrs d, SolveArgs a) {
-  constexpr uint32_t kCompute = kPgsThreads - 32;      // solving threads; the last warp stages
-  constexpr uint32_t kProducer = kCompute;             // the staging thread (lane 0 of the last warp)
-  constexpr uint32_t kWave = pgs_wave(kPgsThreads, kPerThread);  // contacts per wave
-  constexpr size_t kStageBytes = stage_bytes(kWave);
+// The persistent solver. The colour order is cut into row tiles of 32
+// contacts, dealt out to the warps in turn. A warp runs through its tiles
+// sweep after sweep without any barrier: rows and impulses arrive in a ring of
+// shared memory (cp.async, or stay there when the ring holds all of the warp's
+// tiles), the particle records of the next tile are read while this one is
+// solved, and a contact waits only for the versions of its two particles. Grid
+// barriers remain around residual checks.
+//
+// What bounds it: on beds of a few thousand tiles the chain of dependent
+// updates (about 2.5 us of L2 round trips and arithmetic from one update of a
+// particle to the next); on the largest beds the L1 data pipe (a record is one
+// wavefront per lane and access) and the rows' DRAM traffic. Measured against
+// the solver this replaced (rows staged by a TMA warp, every colour a
+// barrier between neighbouring CTAs), same box, ms for 100 sweeps: 1M spheres
+// (3.2M contacts) 8.84 against 12.1, 200k 2.88 against 5.76, 50k 1.92 against
+// 3.34; 2000 spheres, 50 sweeps 0.61 against 1.18; 64 beds of 406k spheres in
+// all, 50 sweeps 1.49 against 2.64.
+//  - 16 warps an SM with 128 registers each: 26 warps with 72 registers spill,
+//    and spilling took half of the L1 traffic (1M spheres 17.2 ms).
+//  - Tiles in turn rather than a stretch of slots per warp: every warp gets the
+//    same number (2000 spheres 0.70 against 1.48 ms), and dependent tiles are
+//    a whole colour apart.
+//  - One lane polls while a record is two or more updates away: polling with
+//    every lane of every waiting warp saturates L2 (50k spheres 4.42 against
+//    2.69 ms).
+template <int kThreads, int kPerThread, int kMinBlocks>
+__global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveArgs a) {
+  constexpr int kRing = ring_tiles(kPerThread);  // tiles in a warp's ring
+  constexpr int kAhead = kRing - 1;              // tiles fetched ahead
   if (step_failed(d)) return;
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ unsigned long long full[kStages];
-  __shared__ uint32_t s_lo[2 * TDS_MAX_COLOURS], s_hi[2 * TDS_MAX_COLOURS], s_nw[TDS_MAX_COLOURS];
   __shared__ double s_rn[kResSum], s_rd[kResSum];
-  static_assert(kPgsThreads >= (int)kResSum, "the residual sum needs kResSum threads");
-  __shared__ uint32_t s_mn[kPgsThreads / 32], s_mx[kPgsThreads / 32];
-  __shared__ int s_flag, s_fail, s_gaveup;
-  __shared__ uint32_t s_waves, s_jlo, s_jhi;
+  static_assert(kThreads >= (int)kResSum, "the residual sum needs kResSum threads");
+  __shared__ int s_flag;
   __shared__ uint32_t s_done[TDS_MAX_SCENES / 32], s_done_new[TDS_MAX_SCENES / 32];
-  __shared__ uint32_t s_rmax, s_ndone, s_ndone_check;
+  __shared__ uint32_t s_rmax, s_ndone, s_ndone_check, s_next;
   __shared__ unsigned long long s_acc[2];
   const uint32_t ncol = min(d.ctr[CTR_NCOL], (uint32_t)TDS_MAX_COLOURS);
-  const uint32_t nseg = 2 * ncol;
-  const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t stride = gridDim.x * blockDim.x;
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t warp = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+  const uint32_t nwarps = gridDim.x * (kThreads / 32);
   if (threadIdx.x == 0) {
-    s_waves = 0;
-    s_fail = 0;
-    s_gaveup = 0;  // a wait for a staged wave gave up
-    s_jlo = s_jhi = blockIdx.x;
     s_ndone = 0;
     s_acc[0] = s_acc[1] = 0ull;
   }
   for (uint32_t w = threadIdx.x; w < TDS_MAX_SCENES / 32; w += blockDim.x) s_done[w] = 0u;
   __syncthreads();
-  for (uint32_t g = threadIdx.x; g < nseg; g += blockDim.x) seg_chunk(d, g, s_lo[g], s_hi[g]);
-  __syncthreads();
-  for (uint32_t c = threadIdx.x; c < ncol; c += blockDim.x) {
-    s_nw[c] = waves_of(s_hi[2 * c] - s_lo[2 * c], s_hi[2 * c + 1] - s_lo[2 * c + 1], kWave);
-    atomicAdd(&s_waves, s_nw[c]);
-  }
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < kStages; ++k) mbar_init(&full[k], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  const uint32_t waves_per_sweep = s_waves;
   uint32_t gen = 0;  // grid barriers passed
 
-  if (a.sync) {  // this CTA's touched slot range, then its neighbours
-    uint32_t mn = 0xFFFFFFFFu, mx = 0u;
-    for (uint32_t g = 0; g < nseg; ++g)
-      for (uint32_t p = s_lo[g] + threadIdx.x; p < s_hi[g]; p += blockDim.x) {
-        const uint2 ab = __ldcg(d.p_ab + p);
-        if (ab.x == 0xFFFFFFFFu) continue;  // padding slot
-        mn = min(mn, ab.x);
-        mx = max(mx, ab.x);
-        if (is_dyn(ab.y)) {
-          mn = min(mn, ab.y);
-          mx = max(mx, ab.y);
-        }
-      }
+  // Tiles are numbered in (colour, static?, slot) order and dealt out to the
+  // warps in turn: warp w takes w, w + W, ... Every warp has the same number
+  // of them, whatever the buckets' sizes, and the tiles in work at any time
+  // are consecutive ones, a whole colour (a bed's width) ahead of the tiles
+  // that depend on them. Each warp enters its own tiles in the table.
+  uint32_t total = 0;
+  for (uint32_t g0 = 0; g0 < 2 * ncol; g0 += 32) {
+    const uint32_t g = g0 + lane;
+    const uint32_t s = g < 2 * ncol ? d.bstart[g] : 0u, e = g < 2 * ncol ? d.bend[g] : 0u;
+    const uint32_t T = (e - s + 31u) / 32u;
+    uint32_t incl = T;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-      mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t up = __shfl_up_sync(0xffffffffu, incl, o);
+      if ((int)lane >= o) incl += up;
     }
-    if ((threadIdx.x & 31) == 0) {
-      s_mn[threadIdx.x >> 5] = mn;
-      s_mx[threadIdx.x >> 5] = mx;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < kPgsThreads / 32; ++w) {
-        mn = min(mn, s_mn[w]);
-        mx = max(mx, s_mx[w]);
-      }
-      __stcg(d.rng + 2 * blockIdx.x, mn);
-      __stcg(d.rng + 2 * blockIdx.x + 1, mx);
-      s_mn[0] = mn;
-      s_mx[0] = mx;
-    }
-    if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) return;
-    const uint32_t lo = s_mn[0], hi = s_mx[0];
-    for (uint32_t j = threadIdx.x; j < gridDim.x; j += blockDim.x) {
-      const uint32_t jl = __ldcg(d.rng + 2 * j), jh = __ldcg(d.rng + 2 * j + 1);
-      if (lo <= hi && jl <= jh && max(lo, jl) <= min(hi, jh)) {
-        atomicMin(&s_jlo, j);
-        atomicMax(&s_jhi, j);
-      }
-    }
-    __syncthreads();
+    const uint32_t base = total + incl - T;  // first tile of the bucket
+    for (uint32_t t = (warp + nwarps - base % nwarps) % nwarps; t < T; t += nwarps)
+      d.tiles[base + t] = make_uint2(s + 32u * t, min(32u, e - s - 32u * t) | (g << 8));
+    total += __shfl_sync(0xffffffffu, incl, 31);
   }
-  const uint32_t jlo = s_jlo, jhi = s_jhi;
-  // staged impulses of a wave were written one sweep earlier by this CTA, so
-  // never run further ahead than one sweep's worth of waves
-  const uint32_t ahead = min((uint32_t)kStages, waves_per_sweep);
+  __syncwarp();
+  const uint32_t ntile = warp < total ? (total - warp + nwarps - 1u) / nwarps : 0u;
+  const uint2 *list = d.tiles + warp;
 
-  // v = M^-1 (p + G^T lambda_0), colour by colour (no conflicts inside one)
-  if (a.apply_warm) {
-    for (uint32_t col = 0; col < ncol; ++col) {
-      for (int part = 0; part < 2; ++part) {
-        const uint32_t s = d.bstart[2 * col + part], e = d.bend[2 * col + part];
-        for (uint32_t p = s + tid; p < e; p += stride) {
-          float4 L0 = d.p_la[p];
-          float2 L1 = d.p_lb[p];
-          if (L0.x == 0.f && L0.y == 0.f && L0.z == 0.f && L0.w == 0.f && L1.x == 0.f && L1.y == 0.f)
-            continue;
-          Row r = load_row(d, p);
-          Side A, B;
-          load_pair(d, r, A, B);
-          float3 t1, t2;
-          onb(r.n, t1, t2);
-          apply(r, A, B, L0.x, L0.y * t1 + L0.z * t2, make_float3(L0.w, L1.x, L1.y));
-          store_side(d, r.ab.x, A);
-          if (r.dyn) store_side(d, r.ab.y, B);
-        }
-      }
-      if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) return;
+  const uint32_t ring = smem_u32(smem) + (threadIdx.x >> 5) * (uint32_t)(kRing * kTileBytes);
+  unsigned char *ring_p = smem + (size_t)(threadIdx.x >> 5) * (kRing * kTileBytes);
+  // lane l keeps entry l of the list's current group of 32
+  uint2 ent = lane < ntile ? list[(size_t)lane * nwarps] : make_uint2(0u, 0u);
+  uint32_t group = 0;
+  auto entry = [&](uint32_t j) {
+    if ((j >> 5) != group) {  // lists of more than 32 tiles
+      group = j >> 5;
+      ent = 32u * group + lane < ntile ? list[(size_t)(32u * group + lane) * nwarps] : make_uint2(0u, 0u);
     }
-  }
+    return make_uint2(__shfl_sync(0xffffffffu, ent.x, j & 31u), __shfl_sync(0xffffffffu, ent.y, j & 31u));
+  };
 
-  // producer (thread kProducer): the next wave to stage
-  uint32_t issued = 0, consumed = 0;
-  WaveSeq prod{0, 0, 0xFFFFFFFFu};
-  if (waves_per_sweep > 0 && a.max_iters > 0) {
-    prod.advance(s_nw, ncol, a.max_iters);  // first wave
-    if (threadIdx.x == kProducer)
-      for (uint32_t k = 0; k < ahead && prod.valid(a.max_iters); ++k) {
-        issue_wave(d, prod, s_lo, s_hi, smem + (size_t)(issued % kStages) * kStageBytes,
-                   &full[issued % kStages], kWave);
-        ++issued;
-        prod.advance(s_nw, ncol, a.max_iters);
-      }
-  }
-
-  bool ok = true;
+  const uint32_t warm = a.apply_warm ? 1u : 0u;
+  // The ring holds all of the warp's tiles: they are fetched once, and the
+  // impulses live in it. Otherwise a tile is fetched again every sweep, at
+  // least one tile after its impulses were stored.
+  const bool resident = ntile <= (uint32_t)kRing;
+  const uint32_t stages = resident ? ntile : (uint32_t)kRing;
+  bool dead = false;  // this warp's wait gave up (the error is latched)
   uint32_t it = 0;
-  float resid = -1.f;
+  uint32_t fetch = 0, fst = 0, st = 0;  // next tile to fetch, its ring stage, the current tile's stage
+  auto fetch_next = [&](bool on) {
+    if (on) {
+      const uint2 e = entry(fetch);
+      const uint32_t stage = ring + fst * (uint32_t)kTileBytes;
+      const bool mine = lane < (e.y & 0xFFu);
+      reinterpret_cast<uint32_t *>(ring_p + fst * kTileBytes + kOffIx * 32)[lane] = mine ? e.x + lane : ~0u;
+      if (mine) stage_row(d, e.x + lane, stage, lane);
+      if (++fetch == ntile) fetch = 0;
+      if (++fst == stages) fst = 0;
+    }
+    cp_commit();
+  };
+  for (int k = 0; k < kAhead; ++k) fetch_next(ntile > 0 && (!resident || k < (int)ntile));
+  // The records of a tile are read one tile ahead: whether they hold the
+  // versions it needs is looked at when its turn comes, and only those that
+  // did not are read again.
+  float4 nva, nwa, nvb, nwb;
+  nva = nwa = nvb = nwb = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto load_sides = [&](const unsigned char *stage) {
+    const uint32_t p = reinterpret_cast<const uint32_t *>(stage + kOffIx * 32)[lane];
+    if (p == ~0u) return;
+    const uint2 ab = reinterpret_cast<const uint2 *>(stage + kOffAb * 32)[lane];
+    ld_rec(d.rec + 2 * (size_t)ab.x, nva, nwa);
+    if (is_dyn(ab.y)) {
+      ld_rec(d.rec + 2 * (size_t)ab.y, nvb, nwb);
+    } else {
+      nvb = __ldg(d.p_sv + p);
+      nwb = __ldg(d.p_sw + p);
+    }
+  };
+  cp_wait<kAhead - 1>();
+  if (ntile > 0) load_sides(ring_p);
+
   // residual checks: every `every` sweeps, or (every == 0) where the decay
   // seen so far says the tolerance will be met (see below)
-  __shared__ uint32_t s_next;
   uint32_t next_check = a.every ? a.every : kFirstCheck;
-  float prev_res = -1.f;
+  float resid = -1.f, prev_res = -1.f;
   uint32_t prev_it = 0;
-  while (ok && it < a.max_iters) {
-    for (uint32_t col = 0; col < ncol; ++col) {
-      const uint32_t phase = it * ncol + col + 1u;
-      const bool busy = s_nw[col] > 0;
-      if (a.sync && busy && !neighbour_wait(d, jlo, jhi, phase - 1u, &s_fail)) { ok = false; break; }
-      for (uint32_t w = 0; w < s_nw[col]; ++w) {
-        const uint32_t st = consumed % kStages;
-        unsigned char *stage = smem + (size_t)st * kStageBytes;
-        // a wait for this CTA's own bulk copies (which complete in
-        // microseconds): the fixed limit, not the limit on waits for others
-        // A wait that gives up (the error is latched) skips this wave, and no
-        // thread leaves the loop here: every CTA leaves it together at the
-        // next residual check, whose grid barrier sees the error. The CTA
-        // stages no wave after it; particle indices read from a stage are
-        // checked against the particle count all the same.
-        const bool staged =
-            threadIdx.x < kCompute && mbar_wait(&full[st], (consumed / kStages) & 1u, d.err, TDS_BARRIER_NS);
-        if (!staged && threadIdx.x < kCompute) s_gaveup = 1;  // read by the staging thread after the barrier
-        const uint2 *sab = reinterpret_cast<const uint2 *>(stage + kOffAb * kWave);
-        const float4 *srn = reinterpret_cast<const float4 *>(stage + kOffRn * kWave);
-        const float4 *srq = reinterpret_cast<const float4 *>(stage + kOffRq * kWave);
-        const float2 *srm = reinterpret_cast<const float2 *>(stage + kOffRm * kWave);
-        const float4 *sla = reinterpret_cast<const float4 *>(stage + kOffLa * kWave);
-        const float2 *slb = reinterpret_cast<const float2 *>(stage + kOffLb * kWave);
-        const WaveDesc q = wave_desc(s_lo[2 * col], s_hi[2 * col], s_lo[2 * col + 1], s_hi[2 * col + 1], w, kWave);
-        Side A[kPerThread], B[kPerThread];
-        uint32_t gp[kPerThread];  // colour-order index of each staged contact (or ~0)
-        uint32_t qs[kPerThread];  // its scene, once some scene of a batch has stopped
-        const bool skip_done = s_ndone != 0u;
-        // gathers of every contact of this thread first (disjoint particles)
-#pragma unroll
-        for (int j = 0; j < kPerThread; ++j) {
-          const uint32_t li = j * kCompute + threadIdx.x;
-          gp[j] = !staged ? ~0u
-                  : li < q.n1 ? q.a1 + li : (li >= q.n1e && li < q.n1e + q.n2 ? q.a2 + (li - q.n1e) : ~0u);
-          if (gp[j] != ~0u) {
-            const uint2 ab = sab[li];
-            if (ab.x < a.n && (!is_dyn(ab.y) || ab.y < a.n)) {  // not a padding slot (all ones)
-              if (skip_done) qs[j] = __ldcg(d.sid + ab.x);
-              A[j] = load_side(d, ab.x);
-              if (is_dyn(ab.y)) B[j] = load_side(d, ab.y);
-              else B[j] = Side{f3(d.p_sv[gp[j]]), f3(d.p_sw[gp[j]]), 0.f, 0.f};
-            }
+  uint32_t passes = 0;  // passes done (warm start and sweeps)
+  bool done = a.max_iters == 0 && !warm;
+  while (!done) {
+    const bool warm_pass = passes < warm;
+    const bool skip_done = s_ndone != 0u;
+    uint32_t col = 0;
+    for (uint32_t j = 0; j < ntile && !dead; ++j) {
+      if (!a.sync)  // grid barrier after every colour
+        for (const uint32_t c = entry(j).y >> 9; col < c; ++col)
+          if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) {
+            cp_wait<0>();
+            return;
           }
+      fetch_next(!resident || (passes == 0 && kAhead + j < ntile));
+      cp_wait<kAhead - 1>();  // this tile's rows and the next one's are here
+      unsigned char *stage = ring_p + st * kTileBytes;
+      if (++st == stages) st = 0;
+      const uint32_t p = reinterpret_cast<const uint32_t *>(stage + kOffIx * 32)[lane];
+      const float4 *s_rn = reinterpret_cast<const float4 *>(stage + kOffRn * 32) + lane;
+      const float4 *s_rq = reinterpret_cast<const float4 *>(stage + kOffRq * 32) + lane;
+      const float4 *s_im = reinterpret_cast<const float4 *>(stage + kOffIm * 32) + lane;
+      uint2 ab = make_uint2(0u, TDS_STATIC);
+      bool live = p != ~0u;
+      if (live) {
+        ab = reinterpret_cast<const uint2 *>(stage + kOffAb * 32)[lane];
+        live = !skip_done || !scene_done(s_done, __ldcg(d.sid + ab.x));
+      }
+      const bool dyn = is_dyn(ab.y);
+      float4 *rec_a = d.rec + 2 * (size_t)ab.x, *rec_b = d.rec + 2 * (size_t)ab.y;
+      float4 va = nva, wa = nwa, vb = nvb, wb = nwb;
+      if (ntile > 1) load_sides(ring_p + st * kTileBytes);
+      uint32_t want_a = 0, want_b = 0;
+      bool need_a = live, need_b = live && dyn;
+      Pre pre;
+      if (live) {
+        const uint32_t rk = reinterpret_cast<const uint32_t *>(stage + kOffRk * 32)[lane];
+        want_a = passes * ((rk >> 8) & 0xFFu) + (rk & 0xFFu);
+        want_b = passes * (rk >> 24) + ((rk >> 16) & 0xFFu);
+        // computed while the records are on their way (the empty asm keeps it here)
+        const float4 rn = *s_rn, rq = *s_rq, im = *s_im;
+        Row r;
+        Side A, B;
+        r.n = f3(rn); r.la = rn.w;
+        r.lb = rq.x; r.Sn = rq.z;
+        A.im = im.x; A.iI = im.y; B.im = im.z; B.iI = im.w;
+        pre = prepare_update(r, A, B, a.sig_t, a.sig_r);
+        asm volatile("" : "+f"(pre.iDn), "+f"(pre.iDt), "+f"(pre.iDr), "+f"(pre.t1.x), "+f"(pre.t1.y), "+f"(pre.t1.z),
+                     "+f"(pre.t2.x), "+f"(pre.t2.y), "+f"(pre.t2.z)::"memory");
+      }
+      // Wait for the versions the tile needs (bounded, as every wait). Every
+      // lane that needs one reads again; while some record has two or more
+      // updates to come, only the lane with the most of them polls.
+      unsigned long long t0 = 0;
+      uint32_t lead = 33u;  // the polling lane; 32: every lane has just read, 33: nothing read again yet
+      for (unsigned spins = 0;; ++spins) {
+        uint32_t behind = 0;
+        if (need_a) {
+          need_a = !is_version(va, wa, want_a);
+          if (need_a) behind = max(1u, want_a - __float_as_uint(va.w));
         }
-#pragma unroll
-        for (int j = 0; j < kPerThread; ++j) {
-          const uint32_t li = j * kCompute + threadIdx.x;
-          if (gp[j] != ~0u) {
-            Row r;
-            r.ab = sab[li];
-            if (r.ab.x >= a.n || (is_dyn(r.ab.y) && r.ab.y >= a.n)) continue;  // padding slot
-            if (skip_done && scene_done(s_done, qs[j])) continue;  // its scene met the tolerance
-            const float4 rn = srn[li], rq = srq[li];
-            const float2 rm = srm[li];
-            r.n = f3(rn); r.la = rn.w;
-            r.lb = rq.x; r.qn = rq.y; r.Sn = rq.z; r.fc = rq.w;
-            r.mu = rm.x; r.rmu = rm.y;
-            r.dyn = is_dyn(r.ab.y);
-            float4 L0 = sla[li];
-            float2 L1 = slb[li];
-            pgs_update(r, A[j], B[j], L0, L1, a.sig_t, a.sig_r);
-            store_side(d, r.ab.x, A[j]);
-            if (r.dyn) store_side(d, r.ab.y, B[j]);
-            d.p_la[gp[j]] = L0;
-            d.p_lb[gp[j]] = L1;
-          }
+        if (need_b) {
+          need_b = !is_version(vb, wb, want_b);
+          if (need_b) behind = max(max(behind, 1u), want_b - __float_as_uint(vb.w));
         }
-        // impulses written above are read back by bulk copies one sweep later
-        asm volatile("fence.proxy.async.global;" ::: "memory");
-        __syncthreads();  // the stage is free again
-        ++consumed;
-        // (no more waves once a wait of this CTA has given up: its stage may
-        // still have a copy landing in it)
-        if (threadIdx.x == kProducer && prod.valid(a.max_iters) && !*(volatile int *)&s_gaveup) {
-          issue_wave(d, prod, s_lo, s_hi, smem + (size_t)(issued % kStages) * kStageBytes,
-                     &full[issued % kStages], kWave);
-          ++issued;
-          prod.advance(s_nw, ncol, a.max_iters);
+        if (dead || !__any_sync(0xffffffffu, behind != 0u)) break;
+        if ((spins & 15u) == 15u) {
+          const unsigned long long t = global_ns();
+          if (t0 == 0) t0 = t;
+          else if (t - t0 > d.wait_ns) latch_error(d.err, DEV_ERR_BARRIER);
+          dead = __any_sync(0xffffffffu, *(volatile int32_t *)d.err != 0);
+        }
+        if (lead == 32u) {
+          const uint32_t worst = __reduce_max_sync(0xffffffffu, (min(behind, 0xFFFFFu) << 5) | lane);
+          if (worst >= 64u) lead = worst & 31u;
+        } else if (lead == 33u || __shfl_sync(0xffffffffu, behind, lead) < 2u) {
+          lead = 32u;
+        }
+        if (lead == 32u || lane == lead) {
+          if (need_a) ld_rec(rec_a, va, wa);
+          if (need_b) ld_rec(rec_b, vb, wb);
         }
       }
-      if (!ok) break;
-      if (a.sync) publish(d, phase);
-      else if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) { ok = false; break; }
+      if (live && !dead) {
+        const float4 rn = *s_rn, rq = *s_rq, im = *s_im;
+        const float2 rm = reinterpret_cast<const float2 *>(stage + kOffRm * 32)[lane];
+        float4 &s_la = reinterpret_cast<float4 *>(stage + kOffLa * 32)[lane];
+        float2 &s_lb = reinterpret_cast<float2 *>(stage + kOffLb * 32)[lane];
+        float4 L0 = s_la;
+        float2 L1 = s_lb;
+        Row r;
+        r.n = f3(rn); r.la = rn.w;
+        r.lb = rq.x; r.qn = rq.y; r.Sn = rq.z; r.fc = rq.w;
+        r.mu = rm.x; r.rmu = rm.y;
+        Side A{f3(va), f3(wa), im.x, im.y}, B{f3(vb), f3(wb), im.z, im.w};
+        if (warm_pass) {  // v = M^-1 (p + G^T lambda_0)
+          if (!(L0.x == 0.f && L0.y == 0.f && L0.z == 0.f && L0.w == 0.f && L1.x == 0.f && L1.y == 0.f))
+            apply(r, A, B, L0.x, L0.y * pre.t1 + L0.z * pre.t2, make_float3(L0.w, L1.x, L1.y));
+        } else {
+          pgs_update(r, pre, A, B, L0, L1, a.sig_t, a.sig_r);
+        }
+        st_rec(rec_a, A.v, A.w, want_a + 1u);
+        if (dyn) st_rec(rec_b, B.v, B.w, want_b + 1u);
+        if (!warm_pass) {
+          d.p_la[p] = L0;
+          d.p_lb[p] = L1;
+          if (resident) {
+            s_la = L0;
+            s_lb = L1;
+          }
+        }
+      }
+      if (ntile == 1) load_sides(stage);
     }
-    if (!ok) break;
-    ++it;
-    if (it == a.max_iters || (a.tol > 0.f && it == next_check)) {
-      // the residual reads every contact: all colours of this sweep first
-      if (a.sync && !grid_barrier(d.bar, d.err, gen, d.wait_ns)) { ok = false; break; }
+    if (!a.sync)
+      for (; col < ncol; ++col)
+        if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) {
+          cp_wait<0>();
+          return;
+        }
+    ++passes;
+    if (!warm_pass) ++it;
+    else if (!dead) {
+      done = a.max_iters == 0;
+      continue;
+    }
+    // (a warp whose wait gave up goes straight to the barrier, which sees the
+    // error in every CTA and ends the launch)
+    if (dead || it == a.max_iters || (a.tol > 0.f && it == next_check)) {
+      // the residual reads every contact: all updates of this sweep first
+      if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) {
+        cp_wait<0>();
+        return;
+      }
       // Every scene has its own residual, summed in an order that neither the
       // launch shape nor the other scenes of a batch change: its chunks (its
       // contacts of one bucket, at most TDS_RES_CHUNK of them, consecutive in
@@ -696,16 +634,14 @@ __global__ void __launch_bounds__(kPgsThreads, kMinBlocks) k_pgs(DevPtrs d, Solv
       // from the same values. A scene that met the tolerance stops sweeping
       // and keeps the residual of that check.
       const uint32_t nchunk = d.ctr[CTR_NCHUNK];
-      const uint32_t lane = threadIdx.x & 31u;
-      for (uint32_t ch = tid >> 5; ch < nchunk; ch += stride >> 5) {
+      for (uint32_t ch = warp; ch < nchunk; ch += nwarps) {
         const uint4 cd = __ldcg(d.chunk + ch);
         if (scene_done(s_done, cd.z)) continue;
         double cn = 0.0, cdn = 0.0;
         for (uint32_t q = lane; q < cd.y; q += 32u) {
           const uint32_t p = cd.x + q;
-          Row r = load_row(d, p);
           Side A, B;
-          load_pair(d, r, A, B);
+          const Row r = settled_pair(d, p, A, B);
           resid_terms(r, A, B, __ldcg(d.p_la + p), __ldcg(d.p_lb + p), a.sig_t, a.sig_r, cn, cdn);
         }
 #pragma unroll
@@ -718,7 +654,10 @@ __global__ void __launch_bounds__(kPgsThreads, kMinBlocks) k_pgs(DevPtrs d, Solv
           __stcg(d.dres + 2 * ch + 1, cdn);
         }
       }
-      if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) { ok = false; break; }
+      if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) {
+        cp_wait<0>();
+        return;
+      }
       const uint32_t S = d.nscenes;
       for (uint32_t w = threadIdx.x; w < (S + 31u) / 32u; w += blockDim.x) s_done_new[w] = 0u;
       if (threadIdx.x == 0) s_rmax = 0u;
@@ -806,16 +745,11 @@ __global__ void __launch_bounds__(kPgsThreads, kMinBlocks) k_pgs(DevPtrs d, Solv
       }
       __syncthreads();
       next_check = s_next;
-      if (s_flag) break;
+      done = s_flag || it == a.max_iters;
     }
   }
-  // drain the waves still in flight before the CTA exits (bulk copies of this
-  // CTA's own: a fixed, generous limit, whatever the limit on waits for others)
-  if (threadIdx.x == kProducer)
-    for (uint32_t q = consumed; q < issued; ++q)
-      if (!mbar_wait(&full[q % kStages], (q / kStages) & 1u, d.err, TDS_BARRIER_NS, false)) break;
-  const bool all_ok = __syncthreads_and(ok) != 0;  // every thread of the CTA reaches this point
-  if (blockIdx.x == 0 && all_ok) {
+  cp_wait<0>();
+  if (blockIdx.x == 0) {
     // statistics: the sweeps done (the most any scene did), the largest final
     // residual, and per scene its sweeps x its contacts (the solver's work)
     __syncthreads();
@@ -907,7 +841,7 @@ __global__ void __launch_bounds__(512) k_impact(DevPtrs d, ImpactArgs a) {
           float2 L1 = make_float2(t.x, t.y);
           Side A, B;
           load_pair(d, r, A, B);
-          pgs_update(r, A, B, L0, L1, a.sig_t, a.sig_r);
+          pgs_update(r, prepare_update(r, A, B, a.sig_t, a.sig_r), A, B, L0, L1, a.sig_t, a.sig_r);
           store_side(d, r.ab.x, A);
           if (r.dyn) store_side(d, r.ab.y, B);
           d.p_il[p] = L0;
@@ -967,7 +901,11 @@ __global__ void k_prev_ranges(DevPtrs d, uint32_t n, uint32_t cap) {
 __global__ void k_integrate(DevPtrs d, StepConsts k) {
   if (step_failed(d)) return;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < k.n; i += gridDim.x * blockDim.x) {
-    float4 p = d.pos[i], v = d.pv[2 * i], w = d.pv[2 * i + 1];
+    // the solved velocities come back from the solver's records
+    const float im = d.pv[2 * i].w, iI = d.pv[2 * i + 1].w;
+    float4 p = d.pos[i], v = d.rec[2 * (size_t)i], w = d.rec[2 * (size_t)i + 1];
+    d.pv[2 * i] = make_float4(v.x, v.y, v.z, im);
+    d.pv[2 * i + 1] = make_float4(w.x, w.y, w.z, iI);
     p.x += k.dt * v.x;
     p.y += k.dt * v.y;
     p.z += k.dt * v.z;
@@ -1055,8 +993,12 @@ static inline unsigned grid_for(uint32_t n, unsigned threads, unsigned maxb = 15
   return b < maxb ? b : maxb;
 }
 
-int tds_launch_predict(const DevPtrs &d, const StepConsts &k, cudaStream_t st) {
-  k_predict<<<grid_for(k.n, 256), 256, 0, st>>>(d, k);
+int tds_launch_predict(const DevPtrs &d, const StepConsts &k, int records, cudaStream_t st) {
+  k_predict<<<grid_for(k.n, 256), 256, 0, st>>>(d, k, records);
+  return 1;
+}
+int tds_launch_records(const DevPtrs &d, uint32_t n, cudaStream_t st) {
+  k_records<<<grid_for(n, 256), 256, 0, st>>>(d, n);
   return 1;
 }
 
@@ -1080,12 +1022,11 @@ cudaError_t tds_launch_pgs(const DevPtrs &d, const StepConsts &k, uint32_t max_i
                            uint32_t every, int apply_warm, int blocks, int sync, int shape, cudaStream_t st) {
   SolveArgs a{max_iters, every, tol, k.sig_t, k.sig_r, apply_warm, sync, k.n};
   cudaMemsetAsync(d.bar, 0, 2 * sizeof(uint32_t), st);
-  if (sync) cudaMemsetAsync(d.prog, 0, sizeof(uint32_t) * kProgStride * (size_t)blocks, st);
   DevPtrs dd = d;
   void *args[] = {&dd, &a};
   const int T = kShapes[shape][0];
   return cudaLaunchCooperativeKernel((const void *)kPgsKernels[shape], dim3(blocks), dim3(T), args,
-                                     pgs_smem(pgs_wave(T, kShapes[shape][1])), st);
+                                     pgs_smem(T, kShapes[shape][1]), st);
 }
 
 cudaError_t tds_launch_impact(const DevPtrs &d, const StepConsts &k, float e, float vimp, uint32_t iters,
@@ -1104,7 +1045,7 @@ int tds_pgs_setup() {
   int occ_min = 0;
   for (int i = 0; i < kNumShapes; ++i) {
     const int T = kShapes[i][0];
-    const size_t smem = pgs_smem(pgs_wave(T, kShapes[i][1]));
+    const size_t smem = pgs_smem(T, kShapes[i][1]);
     if (cudaFuncSetAttribute((const void *)kPgsKernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem) != cudaSuccess)
       return 0;

@@ -38,7 +38,7 @@ EXPORTED = ["tds_workspace_bytes", "tds_create_scene", "tds_set_tool_pose", "tds
             "tds_set_recolour_period"]
 
 WARM_COLD, WARM_PREV, WARM_LEARNED = 0, 1, 2
-SHAPES = ((416, 1), (768, 1), (512, 2), (640, 2), (512, 3), (256, 1))  # solver CTA shapes compiled (threads, contacts per thread)
+SHAPES = ((512, 2), (416, 1), (768, 1), (640, 2), (512, 3), (256, 1))  # solver CTA shapes compiled (threads, row tiles in flight per warp)
 
 
 class TdsError(RuntimeError):
@@ -509,9 +509,9 @@ class Scene:
 
     def set_launch_config(self, pgs_blocks: int = 0, pgs_sync: int | None = None, colour_blocks: int = 0,
                           pgs_threads: int = 0, pgs_per_thread: int = 0, wait_limit_us: int = 0):
-        """Solver CTAs, solver sync mode (1 neighbour, 0 grid barrier),
-        colouring CTAs, the solver CTA shape (threads x contacts per
-        thread, one of SHAPES) and the limit of a wait on other CTAs [us];
+        """Solver CTAs, solver sync mode (1 per particle, 0 grid barrier),
+        colouring CTAs, the solver CTA shape (threads x row tiles in flight
+        per warp, one of SHAPES) and the limit of a wait on other CTAs [us];
         0 (or None for the mode) keeps the current value."""
         c = LaunchConfig()
         _check(lib().tds_get_launch_config(self.h, ctypes.byref(c)))
