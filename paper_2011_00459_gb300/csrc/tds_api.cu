@@ -45,7 +45,7 @@ int tds_launch_aggregate(const DevPtrs &d, uint32_t n, const tds_zone *zones, ui
                          double *sums, tds_aggregate *out, cudaStream_t st);
 size_t tds_aggregate_sums_words();
 int tds_launch_coarse_grain(const DevPtrs &d, uint32_t n, const tds_grid &g, int kernel, float R, float *rho,
-                            float *p, float *u, cudaStream_t st);
+                            float *p, float *u, size_t scratch_cells, cudaStream_t st);
 bool tds_grid_valid(const tds_grid *g);
 const void *tds_colour_kernel();
 
@@ -1482,7 +1482,8 @@ tds_status tds_coarse_grain(tds_scene *s, const tds_grid *grid, int32_t kernel, 
     return fail(TDS_ERR_INVALID_ARG, "Gaussian smoothing length must be in (0, 16 l0]");
   tds_status ls = check_latched(s);
   if (ls != TDS_OK) return ls;
-  s->launches += tds_launch_coarse_grain(s->d, s->L.n, *grid, kernel, R, rho, p, u, s->st);
+  s->launches += tds_launch_coarse_grain(s->d, s->L.n, *grid, kernel, R, rho, p, u,
+                                         (size_t)s->L.cap + TDS_ORDER_PAD, s->st);
   CUDA_TRY(cudaGetLastError());
   return TDS_OK;
 }
