@@ -3,11 +3,20 @@
 // centre of mass, velocity, inertia tensor about the centre of mass and the
 // angular velocity I^+ L of the particles it contains. Two passes, as in the
 // definition: (1) membership, M, sum m x, sum m v; (2) the second moments and
-// angular momentum about the centre of mass. FP64 accumulation, reduced warp
-// by warp (see WarpSums).
+// angular momentum about the centre of mass. FP64 accumulation in
+// registers (see LaneSums). What bounds the passes: FP64 issue and its
+// latency (20 and 31 operations a particle). 1M particles, 8 zones: 53 and 68
+// us; with five shuffle steps and additions per component and 32 particles,
+// and FP64 divisions, 146 and 185. k_agg_final 6.8 us against 24.
+#include <cstring>
+
 #include "tds_internal.cuh"
 
 namespace {
+
+struct ZoneTable {  // the zones as a kernel argument
+  tds_zone z[TDS_MAX_ZONES];
+};
 
 constexpr int kAggThreads = 256;
 constexpr int kFirst = 8;   // m, m x (3), m v (3), count
@@ -30,43 +39,72 @@ __device__ __forceinline__ int zone_of(const tds_zone *zones, uint32_t nz, uint3
   return -1;
 }
 
-// Warp-synchronous accumulation of K sums per zone. Each warp walks its own
-// contiguous stretch of slots, 32 consecutive particles per iteration
-// (coalesced). When every particle of the iteration that lies in a zone lies
-// in the same zone (the usual case: slot order is spatial) the warp reduces
-// the K values with shuffles and lane c keeps component c of the running sum
-// of the warp's current zone, flushed into shared memory when the zone
-// changes; iterations that straddle zones add lane by lane.
+// Mass of a particle: the reciprocal of the FP32 record's 1/m. FP64 division
+// costs about twenty FP64 operations, which this GPU issues at a sixty-fourth
+// of the FP32 rate; Newton's iteration r <- r + r (1 - a r) doubles the correct
+// digits of the FP32 reciprocal, to 2^-46 and then to the last bit.
+__device__ __forceinline__ double mass_of(float inv_m) {
+  const double a = (double)inv_m;
+  double r = (double)__frcp_rn(inv_m);
+  r = fma(r, fma(-a, r, 1.0), r);
+  return fma(r, fma(-a, r, 1.0), r);
+}
+
+// Sums of K components per zone. Each warp walks its own contiguous stretch of
+// slots, 32 consecutive particles per iteration (coalesced); each lane keeps
+// the running sums of the zone of its last particle in registers and flushes
+// them into shared memory when its zone changes (rarely: slot order is
+// spatial). At the end of the stretch the lanes of one zone are added by
+// shuffles first.
 template <int K>
-struct WarpSums {
+struct LaneSums {
   int cur = -1;
-  double acc = 0.0;  // lane c < K: component c for zone cur
-  __device__ void flush(double *sh, int lane) {
-    if (cur >= 0 && lane < K && acc != 0.0) atomicAdd(sh + cur * K + lane, acc);
-    acc = 0.0;
-  }
-  __device__ void add(double *sh, int lane, int z, const double (&val)[K]) {
-    const unsigned full = 0xffffffffu;
-    const int zsel = __reduce_max_sync(full, z);
-    if (zsel < 0) return;
-    const bool uniform = __all_sync(full, z < 0 || z == zsel);
-    if (!uniform) {
-      if (z >= 0)
-#pragma unroll
-        for (int c = 0; c < K; ++c)
-          if (val[c] != 0.0) atomicAdd(sh + z * K + c, val[c]);
-      return;
-    }
-    if (zsel != cur) {
-      flush(sh, lane);
-      cur = zsel;
-    }
+  double acc[K] = {};
+  __device__ __forceinline__ void flush(double *sh) {
 #pragma unroll
     for (int c = 0; c < K; ++c) {
-      double t = val[c];
+      if (cur >= 0 && acc[c] != 0.0) atomicAdd(sh + cur * K + c, acc[c]);
+      acc[c] = 0.0;
+    }
+  }
+  // makes z (>= 0) the zone the sums belong to
+  __device__ __forceinline__ void enter(double *sh, int z) {
+    if (z != cur) {
+      flush(sh);
+      cur = z;
+    }
+  }
+  __device__ __forceinline__ void finish(double *sh) {
+    const unsigned full = 0xffffffffu;
+    __syncwarp();
+    const int z = __reduce_max_sync(full, cur);
+    if (!__all_sync(full, cur == z || cur < 0)) {
+      flush(sh);
+      return;
+    }
+    // eight components: each exchange halves the components a lane holds (9
+    // additions instead of 40); the lane's bits
+    // 4, 3, 2 say which it ends with
+    const unsigned lane = threadIdx.x & 31u;
+#pragma unroll
+    for (int h = 4, o = 16; h > 0; h >>= 1, o >>= 1) {
+      const bool up = lane & (unsigned)o;
+#pragma unroll
+      for (int c = 0; c < h; ++c) {
+        const double keep = up ? acc[c + h] : acc[c], send = up ? acc[c] : acc[c + h];
+        acc[c] = keep + __shfl_xor_sync(full, send, o);
+      }
+    }
+    acc[0] += __shfl_xor_sync(full, acc[0], 2);
+    acc[0] += __shfl_xor_sync(full, acc[0], 1);
+    const int c = (lane & 16u ? 4 : 0) + (lane & 8u ? 2 : 0) + (lane & 4u ? 1 : 0);
+    if (z >= 0 && (lane & 3u) == 0u && acc[0] != 0.0) atomicAdd(sh + z * K + c, acc[0]);
+#pragma unroll
+    for (int q = 8; q < K; ++q) {
+      double t = acc[q];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(full, t, o);
-      if (lane == c) acc += t;
+      if (z >= 0 && lane == 0u && t != 0.0) atomicAdd(sh + z * K + q, t);
     }
   }
 };
@@ -87,38 +125,39 @@ __device__ __forceinline__ void warp_stretch(uint32_t n, uint32_t &lo, uint32_t 
   hi = min(n, lo + per);
 }
 
-__global__ void __launch_bounds__(kAggThreads) k_agg_first(DevPtrs d, uint32_t n, const tds_zone *zones,
-                                                           uint32_t nz, uint8_t *zone_id, double *sums) {
+__global__ void __launch_bounds__(kAggThreads) k_agg_first(DevPtrs d, uint32_t n,
+                                                           const __grid_constant__ ZoneTable zones, uint32_t nz,
+                                                           uint8_t *zone_id, double *sums) {
   __shared__ tds_zone sz[TDS_MAX_ZONES];
   __shared__ double sh[TDS_MAX_ZONES * kFirst];
   for (uint32_t q = threadIdx.x; q < nz * sizeof(tds_zone) / 4; q += blockDim.x)
-    reinterpret_cast<uint32_t *>(sz)[q] = reinterpret_cast<const uint32_t *>(zones)[q];
+    reinterpret_cast<uint32_t *>(sz)[q] = reinterpret_cast<const uint32_t *>(zones.z)[q];
   for (uint32_t q = threadIdx.x; q < nz * kFirst; q += blockDim.x) sh[q] = 0.0;
   __syncthreads();
   const int lane = threadIdx.x & 31;
   uint32_t lo, hi;
   warp_stretch(n, lo, hi);
-  WarpSums<kFirst> ws;
+  LaneSums<kFirst> ls;
   for (uint32_t base = lo; base < hi; base += 32) {
     const uint32_t i = base + lane;
-    int z = -1;
-    double val[kFirst] = {};
-    if (i < hi) {
-      const float4 p = d.pos[i];
-      z = p.w > 0.0f ? zone_of(sz, nz, d.sid[i], p) : -1;  // dormant slots belong to no zone
-      zone_id[i] = z < 0 ? 0xFF : (uint8_t)z;
-      if (z >= 0) {
-        const float4 v = d.pv[2 * (size_t)i];
-        const double m = 1.0 / (double)v.w;
-        val[0] = m;
-        val[1] = m * p.x; val[2] = m * p.y; val[3] = m * p.z;
-        val[4] = m * v.x; val[5] = m * v.y; val[6] = m * v.z;
-        val[7] = 1.0;
-      }
-    }
-    ws.add(sh, lane, z, val);
+    if (i >= hi) continue;
+    const float4 p = d.pos[i];
+    const int z = p.w > 0.0f ? zone_of(sz, nz, d.sid[i], p) : -1;  // dormant slots belong to no zone
+    zone_id[i] = z < 0 ? 0xFF : (uint8_t)z;
+    if (z < 0) continue;
+    const float4 v = d.pv[2 * (size_t)i];
+    ls.enter(sh, z);
+    const double m = mass_of(v.w);
+    ls.acc[0] += m;
+    ls.acc[1] = fma(m, (double)p.x, ls.acc[1]);
+    ls.acc[2] = fma(m, (double)p.y, ls.acc[2]);
+    ls.acc[3] = fma(m, (double)p.z, ls.acc[3]);
+    ls.acc[4] = fma(m, (double)v.x, ls.acc[4]);
+    ls.acc[5] = fma(m, (double)v.y, ls.acc[5]);
+    ls.acc[6] = fma(m, (double)v.z, ls.acc[6]);
+    ls.acc[7] += 1.0;
   }
-  ws.flush(sh, lane);
+  ls.finish(sh);
   block_to_global<kFirst>(sh, sums, nz);
 }
 
@@ -136,26 +175,29 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_second(DevPtrs d, uint32_t 
   const int lane = threadIdx.x & 31;
   uint32_t lo, hi;
   warp_stretch(n, lo, hi);
-  WarpSums<kSecond> ws;
+  LaneSums<kSecond> ls;
   for (uint32_t base = lo; base < hi; base += 32) {
     const uint32_t i = base + lane;
-    int z = -1;
-    double val[kSecond] = {};
-    if (i < hi && zone_id[i] != 0xFF) {
-      z = zone_id[i];
-      const float4 p = d.pos[i];
-      const float4 v = d.pv[2 * (size_t)i];
-      const double m = 1.0 / (double)v.w;
-      const double dx = (double)p.x - com[z][0], dy = (double)p.y - com[z][1], dz = (double)p.z - com[z][2];
-      val[0] = m * dx * dx; val[1] = m * dy * dy; val[2] = m * dz * dz;
-      val[3] = m * dx * dy; val[4] = m * dx * dz; val[5] = m * dy * dz;
-      val[6] = m * (dy * v.z - dz * v.y);
-      val[7] = m * (dz * v.x - dx * v.z);
-      val[8] = m * (dx * v.y - dy * v.x);
-    }
-    ws.add(sh, lane, z, val);
+    const int z = i < hi ? zone_id[i] : 0xFF;
+    if (z == 0xFF) continue;
+    const float4 p = d.pos[i];
+    const float4 v = d.pv[2 * (size_t)i];
+    ls.enter(sh, z);
+    const double m = mass_of(v.w);
+    const double dx = (double)p.x - com[z][0], dy = (double)p.y - com[z][1], dz = (double)p.z - com[z][2];
+    const double vx = (double)v.x, vy = (double)v.y, vz = (double)v.z;
+    const double mx = m * dx, my = m * dy, mz = m * dz;
+    ls.acc[0] = fma(mx, dx, ls.acc[0]);
+    ls.acc[1] = fma(my, dy, ls.acc[1]);
+    ls.acc[2] = fma(mz, dz, ls.acc[2]);
+    ls.acc[3] = fma(mx, dy, ls.acc[3]);
+    ls.acc[4] = fma(mx, dz, ls.acc[4]);
+    ls.acc[5] = fma(my, dz, ls.acc[5]);
+    ls.acc[6] = fma(my, vz, fma(-mz, vy, ls.acc[6]));
+    ls.acc[7] = fma(mz, vx, fma(-mx, vz, ls.acc[7]));
+    ls.acc[8] = fma(mx, vy, fma(-my, vx, ls.acc[8]));
   }
-  ws.flush(sh, lane);
+  ls.finish(sh);
   block_to_global<kSecond>(sh, sums, nz);
 }
 
@@ -207,6 +249,10 @@ __global__ void k_agg_final(uint32_t nz, const double *first, const double *seco
       o.com[a] = F[1 + a] / M;
       o.vel[a] = F[4 + a] / M;
     }
+    if (o.count == 1u) {  // one point: no extent, no spin (its centre of mass is its position to rounding only)
+      out[z] = o;
+      return;
+    }
     // I = tr(S) 1 - S with S the second moment about the centre of mass
     const double tr = S[0] + S[1] + S[2];
     double I[3][3] = {{tr - S[0], -S[3], -S[4]}, {-S[3], tr - S[1], -S[5]}, {-S[4], -S[5], tr - S[2]}};
@@ -215,14 +261,28 @@ __global__ void k_agg_final(uint32_t nz, const double *first, const double *seco
     // the momentum about the centre of mass of the velocities relative to v_A
     // equals sum m dx x v, since sum m dx = 0
     const double L[3] = {S[6], S[7], S[8]};
-    double V[3][3];
-    jacobi3(I, V);
-    const double lam[3] = {I[0][0], I[1][1], I[2][2]};
-    const double lmax = fmax(fabs(lam[0]), fmax(fabs(lam[1]), fabs(lam[2])));
-    for (int k = 0; k < 3; ++k) {
-      if (!(fabs(lam[k]) > 1e-12 * lmax)) continue;  // pseudo-inverse: skip null directions
-      const double proj = (V[0][k] * L[0] + V[1][k] * L[1] + V[2][k] * L[2]) / lam[k];
-      for (int a = 0; a < 3; ++a) o.omega[a] += proj * V[a][k];
+    // omega = I^+ L. det I = l1 l2 l3 <= lmin tr^2, so with det > 1e-10 tr^3
+    // every eigenvalue is far above the pseudo-inverse's cut (1e-12 of the
+    // largest) and I^+ is the inverse, I^-1 L = adj(I) L / det I; the
+    // decomposition (about 20 us of dependent FP64 divisions) is for the rest.
+    const double c00 = I[1][1] * I[2][2] - I[1][2] * I[1][2], c01 = I[0][2] * I[1][2] - I[0][1] * I[2][2],
+                 c02 = I[0][1] * I[1][2] - I[0][2] * I[1][1], c11 = I[0][0] * I[2][2] - I[0][2] * I[0][2],
+                 c12 = I[0][1] * I[0][2] - I[0][0] * I[1][2], c22 = I[0][0] * I[1][1] - I[0][1] * I[0][1];
+    const double det = I[0][0] * c00 + I[0][1] * c01 + I[0][2] * c02, trI = I[0][0] + I[1][1] + I[2][2];
+    if (det > 1e-10 * trI * trI * trI) {
+      o.omega[0] = (c00 * L[0] + c01 * L[1] + c02 * L[2]) / det;
+      o.omega[1] = (c01 * L[0] + c11 * L[1] + c12 * L[2]) / det;
+      o.omega[2] = (c02 * L[0] + c12 * L[1] + c22 * L[2]) / det;
+    } else {
+      double V[3][3];
+      jacobi3(I, V);
+      const double lam[3] = {I[0][0], I[1][1], I[2][2]};
+      const double lmax = fmax(fabs(lam[0]), fmax(fabs(lam[1]), fabs(lam[2])));
+      for (int k = 0; k < 3; ++k) {
+        if (!(fabs(lam[k]) > 1e-12 * lmax)) continue;  // pseudo-inverse: skip null directions
+        const double proj = (V[0][k] * L[0] + V[1][k] * L[1] + V[2][k] * L[2]) / lam[k];
+        for (int a = 0; a < 3; ++a) o.omega[a] += proj * V[a][k];
+      }
     }
   }
   out[z] = o;
@@ -236,12 +296,16 @@ int tds_launch_aggregate(const DevPtrs &d, uint32_t n, const tds_zone *zones, ui
   cudaMemsetAsync(sums, 0, sizeof(double) * TDS_MAX_ZONES * (kFirst + kSecond), st);
   int sms = 152, dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // 8 blocks per SM (the warps walk stretches of ~n / (64 SMs) slots), fewer
-  // for small n so that every warp has at least 128 slots
+  // three blocks per SM (1, 2, 3, 4, 6: 156, 122, 121, 129, 137 us for both
+  // passes over 1M particles; the longer a warp's stretch, the fewer reductions
+  // at its end), fewer for small n so that every
+  // warp has at least 128 slots
   uint32_t blocks = (n + 128u * (kAggThreads / 32) - 1) / (128u * (kAggThreads / 32));
   if (blocks < 1) blocks = 1;
-  if (blocks > (uint32_t)(8 * sms)) blocks = 8 * sms;
-  k_agg_first<<<blocks, kAggThreads, 0, st>>>(d, n, zones, nz, zone_id, first);
+  if (blocks > (uint32_t)(3 * sms)) blocks = 3 * sms;
+  ZoneTable table;
+  std::memcpy(table.z, zones, sizeof(tds_zone) * nz);
+  k_agg_first<<<blocks, kAggThreads, 0, st>>>(d, n, table, nz, zone_id, first);
   k_agg_second<<<blocks, kAggThreads, 0, st>>>(d, n, nz, zone_id, first, second);
   k_agg_final<<<1, TDS_MAX_ZONES, 0, st>>>(nz, first, second, out);
   return 3;

@@ -114,8 +114,7 @@ struct Layout {
 };
 
 struct Extra {  // workspace regions that are not kernel pointers of DevPtrs
-  tds_zone *zones = nullptr;       // aggregate bodies: zones, per-particle zone, sums, results
-  uint8_t *zone_id = nullptr;
+  uint8_t *zone_id = nullptr;      // aggregate bodies: per-particle zone, sums, results
   double *agg_sums = nullptr;
   tds_aggregate *agg_out = nullptr;
   float *heights = nullptr;
@@ -467,7 +466,6 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
   x.packed = c.take<unsigned char>(tds_mlp_packed_bytes());
   x.params = c.take<float>(tds_mlp_params());
   x.heights = c.take<float>(L.nheights);
-  x.zones = c.take<tds_zone>(TDS_MAX_ZONES);
   x.zone_id = c.take<uint8_t>(n);
   x.agg_sums = c.take<double>(tds_aggregate_sums_words());
   x.agg_out = c.take<tds_aggregate>(TDS_MAX_ZONES);
@@ -1464,8 +1462,7 @@ tds_status tds_aggregate_bodies(tds_scene *s, const tds_zone *zones, uint32_t co
   tds_status ls = check_latched(s);
   if (ls != TDS_OK) return ls;
   if (count == 0) return TDS_OK;
-  CUDA_TRY(cudaMemcpyAsync(s->x.zones, zones, sizeof(tds_zone) * count, cudaMemcpyHostToDevice, s->st));
-  s->launches += tds_launch_aggregate(s->d, s->L.n, s->x.zones, count, s->x.zone_id, s->x.agg_sums,
+  s->launches += tds_launch_aggregate(s->d, s->L.n, zones, count, s->x.zone_id, s->x.agg_sums,
                                       s->x.agg_out, s->st);
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaMemcpyAsync(out, s->x.agg_out, sizeof(tds_aggregate) * count, cudaMemcpyDeviceToHost, s->st));
