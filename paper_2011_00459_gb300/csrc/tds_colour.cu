@@ -380,12 +380,13 @@ __global__ void __launch_bounds__(1024) k_scene_chunks(DevPtrs d) {
 
 int tds_launch_colouring(const DevPtrs &d, uint32_t n, uint32_t cap, int coop_blocks,
                          int coop_threads, cudaStream_t st) {
+  int scans = 0;
   unsigned gc = (cap + 255) / 256;
   if (gc > 152 * 16) gc = 152 * 16;
   if (gc == 0) gc = 1;
   cudaMemsetAsync(d.inc_cnt, 0, sizeof(uint32_t) * (n + 1), st);
   k_inc_count<<<gc, 256, 0, st>>>(d);
-  tds_scan_exclusive(d.inc_cnt, d.inc_start, n, d.scan_tmp, st);
+  scans += tds_scan_exclusive(d.inc_cnt, d.inc_start, n, d.scan_tmp, st);
   cudaMemcpyAsync(d.inc_cursor, d.inc_start, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st);
   k_inc_fill<<<gc, 256, 0, st>>>(d);
   cudaMemsetAsync(d.ctr + CTR_FCOUNT, 0, 3 * sizeof(uint32_t), st);
@@ -397,20 +398,21 @@ int tds_launch_colouring(const DevPtrs &d, uint32_t n, uint32_t cap, int coop_bl
   cudaLaunchCooperativeKernel((const void *)k_colour_rounds, dim3(coop_blocks), dim3(coop_threads),
                               args, 0, st);
   k_colour_masks<<<(n + 255) / 256 < 152 * 16 ? (n + 255) / 256 : 152 * 16, 256, 0, st>>>(d, n);
-  return 9;
+  return 5 + scans;
 }
 
 // Contact rows (and initial impulses) into the padded colour order.
 int tds_launch_bucketing(const DevPtrs &d, uint32_t cap, cudaStream_t st) {
+  int scans = 0;
   k_bucket_hist<<<d.ntiles, 256, 0, st>>>(d);
-  tds_scan_exclusive(d.tile_hist, d.tile_off, TDS_NBUCKETS * d.ntiles, d.scan_tmp, st);
+  scans += tds_scan_exclusive(d.tile_hist, d.tile_off, TDS_NBUCKETS * d.ntiles, d.scan_tmp, st);
   k_bucket_starts<<<1, 32, 0, st>>>(d);
   cudaMemsetAsync(d.order, 0xFF, sizeof(uint32_t) * ((size_t)cap + TDS_ORDER_PAD), st);
   cudaMemsetAsync(d.p_ab, 0xFF, sizeof(uint2) * ((size_t)cap + TDS_ORDER_PAD), st);  // padding sentinel
   if (d.nscenes > 1) cudaMemsetAsync(d.scq_cnt, 0, sizeof(uint32_t) * (size_t)d.nscenes * TDS_NBUCKETS, st);
   k_bucket_scatter<<<d.ntiles, 256, 0, st>>>(d);
   k_scene_chunks<<<1, 1024, 0, st>>>(d);
-  return 5;
+  return 4 + scans;
 }
 
 const void *tds_colour_kernel() { return (const void *)k_colour_rounds; }

@@ -202,13 +202,14 @@ unsigned blocks_for(uint32_t n) {
 }  // namespace
 
 int tds_launch_cut(const DevPtrs &d, const StepConsts &k, float *heights, uint32_t nh, cudaStream_t st) {
+  int scans = 0;
   cudaMemsetAsync(d.ctr + CTR_SPAWN, 0, sizeof(uint32_t), st);
   k_dorm_flags<<<blocks_for(k.n), 256, 0, st>>>(d, k.n);
-  tds_scan_exclusive(d.dorm_rank, d.dorm_rank, k.n, d.scan_tmp, st);
+  scans += tds_scan_exclusive(d.dorm_rank, d.dorm_rank, k.n, d.scan_tmp, st);
   k_dorm_list<<<blocks_for(k.n), 256, 0, st>>>(d, k.n);
   k_cut<<<blocks_for(nh), 256, 0, st>>>(d, k, heights, nh);
   k_cut_count<<<blocks_for(nh), 256, 0, st>>>(d, k, heights, nh);
-  tds_scan_exclusive(d.hf_cnt, d.hf_rank, nh, d.scan_tmp, st);
+  scans += tds_scan_exclusive(d.hf_cnt, d.hf_rank, nh, d.scan_tmp, st);
   k_cut_write<<<blocks_for(nh), 256, 0, st>>>(d, k, heights, nh);
-  return 11;
+  return 5 + scans;
 }

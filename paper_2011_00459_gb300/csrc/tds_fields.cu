@@ -299,12 +299,12 @@ int tds_launch_coarse_grain(const DevPtrs &d, uint32_t n, const tds_grid &g, int
     b.v = b.x + n;
     cudaMemsetAsync(b.count, 0, sizeof(uint32_t) * (nvox + 1), st);
     k_cg_bin<<<grid_blocks(n), kThreads, 0, st>>>(d, n, g, b);
-    tds_scan_exclusive(b.count, b.count, (uint32_t)nvox, tmp, st);
+    const int scans = tds_scan_exclusive(b.count, b.count, (uint32_t)nvox, tmp, st);
     k_cg_place<<<grid_blocks(n), kThreads, 0, st>>>(d, n, R, b);
     const int reach = (int)floorf(3.0f * R / g.l0 + 0.5f + 1e-3f), span = 2 * reach + 1;
     k_cg_gather<<<std::min(grid_blocks(nvox * 32), 152 * kGatherBlocks), kThreads, sizeof(uint32_t) * span * span, st>>>(
         g, R, reach, b, (uint32_t)nvox, rho, p, u);
-    return 6;
+    return 3 + scans;
   }
   cudaMemsetAsync(rho, 0, sizeof(float) * nvox, st);
   cudaMemsetAsync(p, 0, sizeof(float) * 3 * nvox, st);

@@ -321,7 +321,7 @@ __device__ __forceinline__ bool grid_barrier(uint32_t *bar, int32_t *err, uint32
   return s_ok != 0;
 }
 
-// Host-side launchers implemented in the .cu files.
-void tds_scan_exclusive(const uint32_t *in, uint32_t *out, uint32_t m, uint32_t *tmp,
+// Host-side launchers implemented in the .cu files (the scan returns its launches).
+int tds_scan_exclusive(const uint32_t *in, uint32_t *out, uint32_t m, uint32_t *tmp,
                         cudaStream_t st);
 size_t tds_scan_tmp_words(uint32_t m);
