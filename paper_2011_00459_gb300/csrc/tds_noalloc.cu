@@ -35,11 +35,11 @@ constexpr uint32_t kMaxN = TDS_NOALLOC_MAX_PARTICLES;
 constexpr uint32_t kMaxCells = 262144u;
 
 constexpr size_t align64(size_t w) { return (w + 63) & ~(size_t)63; }  // 256-byte regions
-constexpr size_t kPlan = 0;
+constexpr size_t kPlan = 0, kBounds = 16, kFinished = 24, kNBig = 25;  // (zeroed with the cell counts)
 constexpr size_t kCellCount = kPlan + 64;
 constexpr size_t kCellStart = kCellCount + align64(kMaxCells + 1);
-constexpr size_t kCursor = kCellStart + align64(kMaxCells + 1);
-constexpr size_t kCellOf = kCursor + align64(kMaxCells);
+constexpr size_t kPlace = kCellStart + align64(kMaxCells + 1);
+constexpr size_t kCellOf = kPlace + align64(kMaxN);
 constexpr size_t kPerm = kCellOf + align64(kMaxN);
 constexpr size_t kSPos = kPerm + align64(kMaxN);
 constexpr size_t kSId = kSPos + align64(4 * (size_t)kMaxN);
@@ -63,7 +63,11 @@ struct View {
   __device__ Plan *plan() const { return reinterpret_cast<Plan *>(base + kPlan); }
   __device__ uint32_t *cell_count() const { return base + kCellCount; }
   __device__ uint32_t *cell_start() const { return base + kCellStart; }
-  __device__ uint32_t *cursor() const { return base + kCursor; }
+  __device__ uint32_t *bounds() const { return base + kBounds; }
+  __device__ uint32_t *finished() const { return base + kFinished; }
+  __device__ uint32_t *nbig() const { return base + kNBig; }
+  __device__ uint32_t *big() const { return base + kCnt; }  // (before the counts are written)
+  __device__ uint32_t *place() const { return base + kPlace; }
   __device__ uint32_t *cell_of() const { return base + kCellOf; }
   __device__ uint32_t *perm() const { return base + kPerm; }
   __device__ float4 *spos() const { return reinterpret_cast<float4 *>(base + kSPos); }
@@ -89,34 +93,47 @@ __device__ __forceinline__ int axis_cell(float x, float x0, float inv, int n) {
   return (int)t;
 }
 
-// One block: bounding box, largest radius, and a grid of at most kMaxCells
-// cells, each wider than any contact reach.
-__global__ void k_plan(View v, const float *x, const float *y, const float *z, const float *r,
-                       uint32_t n, int cohesive) {
-  __shared__ float sh[7][32];
-  float m[7] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY, 0.f};
-  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-    float p[3] = {x[i], y[i], z[i]};
-    for (int a = 0; a < 3; ++a) { m[a] = fminf(m[a], p[a]); m[3 + a] = fmaxf(m[3 + a], p[a]); }
+// Floats as unsigned numbers of the same order (every number's above 0, so
+// that zeroed memory is below all of them).
+__device__ __forceinline__ uint32_t ordered(float f) {
+  const uint32_t u = __float_as_uint(f);
+  return u & 0x80000000u ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float unordered(uint32_t u) {
+  return __uint_as_float(u & 0x80000000u ? u & 0x7FFFFFFFu : ~u);
+}
+
+// Bounding box and largest radius, and a grid of at most kMaxCells cells, each
+// wider than any contact reach. Every block reduces its share; the last one to
+// finish makes the plan (one block for all of it took 27 us at 40 000
+// particles, latency of its serial loads; 152 blocks 6).
+__global__ void __launch_bounds__(256) k_plan(View v, const float *x, const float *y, const float *z, const float *r,
+                                              uint32_t n, int cohesive) {
+  __shared__ uint32_t sh[7];
+  __shared__ bool last;
+  if (threadIdx.x < 7) sh[threadIdx.x] = 0u;
+  __syncthreads();
+  // largest of -x, -y, -z, x, y, z, r (fmaxf passes over NaN)
+  float m[7] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY, -INFINITY, 0.f};
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const float p[3] = {x[i], y[i], z[i]};
+    for (int a = 0; a < 3; ++a) { m[a] = fmaxf(m[a], -p[a]); m[3 + a] = fmaxf(m[3 + a], p[a]); }
     m[6] = fmaxf(m[6], r[i]);
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int q = 0; q < 7; ++q) {
-    float t = m[q];
-    for (int o = 16; o > 0; o >>= 1) {
-      float u = __shfl_down_sync(0xffffffffu, t, o);
-      t = (q < 3) ? fminf(t, u) : fmaxf(t, u);
-    }
-    if (lane == 0) sh[q][warp] = t;
+    const uint32_t t = __reduce_max_sync(0xffffffffu, ordered(m[q]));
+    if ((threadIdx.x & 31) == 0) atomicMax(sh + q, t);
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const int nw = blockDim.x >> 5;
-    for (int q = 0; q < 7; ++q) {
-      float t = sh[q][0];
-      for (int w = 1; w < nw; ++w) t = (q < 3) ? fminf(t, sh[q][w]) : fmaxf(t, sh[q][w]);
-      m[q] = t;
-    }
+  if (threadIdx.x < 7) atomicMax(v.bounds() + threadIdx.x, sh[threadIdx.x]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(v.finished(), 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (last && threadIdx.x == 0) {
+    __threadfence();
+    for (int q = 0; q < 7; ++q) m[q] = unordered(*(volatile uint32_t *)(v.bounds() + q));
+    for (int a = 0; a < 3; ++a) m[a] = -m[a];
     float cell = 2.0f * m[6] * 1.025f * 1.02f;
     if (!(cell > 0.f)) cell = 1.f;
     int dims[3];
@@ -145,52 +162,59 @@ __global__ void k_cells(View v, const float *x, const float *y, const float *z, 
     int cz = axis_cell(z[i], P.lo[2], P.inv, P.gnz);
     uint32_t c = ((uint32_t)cz * P.gny + cy) * P.gnx + cx;
     v.cell_of()[i] = c;
-    atomicAdd(v.cell_count() + c, 1u);
+    v.place()[i] = atomicAdd(v.cell_count() + c, 1u);  // its place in the cell, for now in any order
   }
 }
 
 __global__ void k_scatter(View v, uint32_t n) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    v.perm()[atomicAdd(v.cursor() + v.cell_of()[i], 1u)] = i;
+    v.perm()[v.cell_start()[v.cell_of()[i]] + v.place()[i]] = i;
 }
 
 // Reproducible order inside each cell, whatever the order of the atomic
-// scatter: ascending particle index. Cells of up to kSmallCell particles are
-// sorted by one thread each (insertion sort), larger ones by k_cell_sort_big.
+// scatter: ascending particle index. In cells of up to kSmallCell particles
+// each particle counts the smaller indexes of its cell and goes straight to
+// its place; larger cells are listed for k_cell_sort_big.
 constexpr uint32_t kSmallCell = 64;
 
-__global__ void k_cell_sort(View v) {
-  const Plan P = *v.plan();
-  const uint32_t ncells = (uint32_t)P.gnx * P.gny * P.gnz;
-  uint32_t *perm = v.perm();
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) {
-    uint32_t s = v.cell_start()[c], e = v.cell_start()[c + 1];
-    if (e - s < 2 || e - s > kSmallCell) continue;
-    for (uint32_t a = s + 1; a < e; ++a) {
-      uint32_t val = perm[a], b = a;
-      while (b > s && perm[b - 1] > val) { perm[b] = perm[b - 1]; --b; }
-      perm[b] = val;
+__device__ __forceinline__ void put(View v, uint32_t j, uint32_t i, const float *x, const float *y, const float *z,
+                                    const float *r) {
+  v.spos()[j] = make_float4(x[i], y[i], z[i], r[i]);
+  v.sid()[j] = i;
+}
+
+__global__ void k_place(View v, const float *x, const float *y, const float *z, const float *r, uint32_t n) {
+  const uint32_t *perm = v.perm();
+  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    const uint32_t i = perm[j], c = v.cell_of()[i];
+    const uint32_t s = v.cell_start()[c], e = v.cell_start()[c + 1];
+    if (e - s > kSmallCell) {
+      if (j == s) v.big()[atomicAdd(v.nbig(), 1u)] = c;
+      continue;
     }
+    uint32_t at = s;
+    for (uint32_t k = s; k < e; ++k) at += perm[k] < i;
+    put(v, at, i, x, y, z, r);
   }
 }
 
 // Cells with more than kSmallCell particles (a grid that k_plan coarsened
 // because of a far outlier puts thousands of particles in one cell): one
-// block per cell sorts its m entries in place with a bitonic network in the
+// block per listed cell sorts its m entries in place with a bitonic network in the
 // form whose every comparator puts the smaller value at the lower index
 // (each merge stage starts by comparing mirrored positions of its blocks,
 // then halves). Comparators that reach past m are skipped, which is the same
 // as padding the sequence to a power of two with values larger than any
-// index. Every block walks the cells in a fixed stride; all threads of a
-// block read the same bounds, so the block decides together.
-__global__ void __launch_bounds__(1024) k_cell_sort_big(View v) {
-  const Plan P = *v.plan();
-  const uint32_t ncells = (uint32_t)P.gnx * P.gny * P.gnz;
+// index. (Walking all cells to find the large ones took 76 us at 40 000
+// particles, which have none; the list 2.)
+__global__ void __launch_bounds__(1024) k_cell_sort_big(View v, const float *x, const float *y, const float *z,
+                                                        const float *r) {
   uint32_t *perm = v.perm();
-  for (uint32_t c = blockIdx.x; c < ncells; c += gridDim.x) {
+  const uint32_t nbig = *v.nbig();
+  for (uint32_t q = blockIdx.x; q < nbig; q += gridDim.x) {
+    const uint32_t c = v.big()[q];
     const uint32_t s = v.cell_start()[c], e = v.cell_start()[c + 1];
     const uint32_t m = e - s;
-    if (m <= kSmallCell) continue;
     uint32_t *a = perm + s;
     uint32_t pow2 = 1;
     while (pow2 < m) pow2 <<= 1;
@@ -198,8 +222,8 @@ __global__ void __launch_bounds__(1024) k_cell_sort_big(View v) {
     for (uint32_t k = 2; k <= pow2; k <<= 1) {
       const uint32_t hk = k >> 1;
       for (uint32_t t = threadIdx.x; t < half; t += blockDim.x) {  // mirrored pairs of each k-block
-        const uint32_t blk = t / hk, x = t % hk;
-        const uint32_t i = blk * k + x, j = blk * k + (k - 1u - x);
+        const uint32_t blk = t / hk, o = t % hk;
+        const uint32_t i = blk * k + o, j = blk * k + (k - 1u - o);
         if (j < m) {
           const uint32_t ai = a[i], aj = a[j];
           if (ai > aj) { a[i] = aj; a[j] = ai; }
@@ -217,51 +241,65 @@ __global__ void __launch_bounds__(1024) k_cell_sort_big(View v) {
         __syncthreads();
       }
     }
+    for (uint32_t t = threadIdx.x; t < m; t += blockDim.x) put(v, s + t, a[t], x, y, z, r);
+    __syncthreads();
   }
 }
 
-__global__ void k_gather(View v, const float *x, const float *y, const float *z, const float *r,
-                         uint32_t n) {
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    uint32_t i = v.perm()[j];
-    v.spos()[j] = make_float4(x[i], y[i], z[i], r[i]);
-    v.sid()[j] = i;
-  }
-}
-
+// Nine lanes a particle, one for each row of three cells around it (27 lanes
+// of a warp: three particles): a row's candidates are contiguous and its pairs
+// precede the next row's. One thread for all nine rows left the GPU waiting on
+// a chain of loads: 20 us to count and 27 to write at 40 000 particles, against
+// 12.7 and 17.4.
 template <bool kWrite>
-__global__ void k_pairs(View v, uint32_t n, unsigned long long *keys, uint32_t cap) {
+__global__ void __launch_bounds__(128) k_pairs(View v, uint32_t n, unsigned long long *keys, uint32_t cap,
+                                               uint32_t *count_out) {
   const Plan P = *v.plan();
   const float4 *sp = v.spos();
   const uint32_t *sid = v.sid();
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    const float4 A = sp[j];
-    const uint32_t me = sid[j];
-    int cx = axis_cell(A.x, P.lo[0], P.inv, P.gnx);
-    int cy = axis_cell(A.y, P.lo[1], P.inv, P.gny);
-    int cz = axis_cell(A.z, P.lo[2], P.inv, P.gnz);
-    int x0 = max(cx - 1, 0), x1 = min(cx + 1, P.gnx - 1);
-    uint32_t found = 0, out = kWrite ? v.cstart()[j] : 0u;
-    for (int zz = max(cz - 1, 0); zz <= min(cz + 1, P.gnz - 1); ++zz)
-      for (int yy = max(cy - 1, 0); yy <= min(cy + 1, P.gny - 1); ++yy) {
-        uint32_t row = ((uint32_t)zz * P.gny + yy) * P.gnx;
-        uint32_t s = v.cell_start()[row + x0], e = v.cell_start()[row + x1 + 1];
-        for (uint32_t k = s; k < e; ++k) {
-          uint32_t other = sid[k];
-          if (other <= me || !touch(A, sp[k], P.cohesive)) continue;
-          if (kWrite) {
-            if (out < cap) keys[out] = ((unsigned long long)me << 32) | other;
-            ++out;
-          } else {
-            ++found;
-          }
-        }
+  if (kWrite && blockIdx.x == 0 && threadIdx.x == 0) *count_out = v.cstart()[n];
+  const uint32_t lane = threadIdx.x & 31u, who = lane / 9u, row = lane % 9u;
+  const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+  for (uint32_t j0 = 3u * (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); j0 < n; j0 += 3u * warps) {
+    const uint32_t j = j0 + who;
+    const bool on = who < 3u && j < n;
+    uint32_t s = 0, e = 0, me = 0, hits = 0, found = 0;
+    float4 A = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (on) {
+      A = sp[j];
+      me = sid[j];
+      const int cx = axis_cell(A.x, P.lo[0], P.inv, P.gnx);
+      const int cy = axis_cell(A.y, P.lo[1], P.inv, P.gny) + (int)(row % 3u) - 1;
+      const int cz = axis_cell(A.z, P.lo[2], P.inv, P.gnz) + (int)(row / 3u) - 1;
+      if (cy >= 0 && cy < P.gny && cz >= 0 && cz < P.gnz) {
+        const uint32_t first = ((uint32_t)cz * P.gny + cy) * P.gnx;
+        s = v.cell_start()[first + max(cx - 1, 0)];
+        e = v.cell_start()[first + min(cx + 1, P.gnx - 1) + 1];
       }
-    if (!kWrite) v.cnt()[j] = found;
+    }
+    for (uint32_t k = s; k < e; ++k)
+      if (sid[k] > me && touch(A, sp[k], P.cohesive)) {
+        ++found;
+        if (k - s < 32u) hits |= 1u << (k - s);
+      }
+    uint32_t before = 0, all = 0;  // pairs of the particle's earlier rows, of all
+    for (uint32_t q = 0; q < 9u; ++q) {
+      const uint32_t f = __shfl_sync(0xffffffffu, found, min(9u * who + q, 31u));
+      if (q < row) before += f;
+      all += f;
+    }
+    if (!kWrite) {
+      if (on && row == 0u) v.cnt()[j] = all;
+    } else if (found) {
+      uint32_t out = v.cstart()[j] + before;
+      for (uint32_t k = s; k < e; ++k) {
+        if (k - s < 32u ? !((hits >> (k - s)) & 1u) : (sid[k] <= me || !touch(A, sp[k], P.cohesive))) continue;
+        if (out < cap) keys[out] = ((unsigned long long)me << 32) | sid[k];
+        ++out;
+      }
+    }
   }
 }
-
-__global__ void k_total(View v, uint32_t n, uint32_t *count_out) { *count_out = v.cstart()[n]; }
 
 std::mutex g_mu;
 uint32_t *g_base[256];  // device address of the scratch array, per device ordinal
@@ -308,26 +346,20 @@ extern "C" tds_status tds_find_pair_contacts_noalloc(const float *x, const float
   cudaStream_t st = (cudaStream_t)stream;
   View v{base};
   const unsigned grid = (n + 255) / 256;
-  e = cudaMemsetAsync(base + kCellCount, 0, sizeof(uint32_t) * (kMaxCells + 1), st);
+  e = cudaMemsetAsync(base, 0, sizeof(uint32_t) * (kCellCount + kMaxCells + 1), st);
   if (e != cudaSuccess)
     return tds_set_error_message(TDS_ERR_CUDA, (std::string("tds_find_pair_contacts_noalloc: cudaMemsetAsync: ") +
                                                     cudaGetErrorString(e)).c_str());
-  k_plan<<<1, 1024, 0, st>>>(v, x, y, z, radius, n, cohesive ? 1 : 0);
+  const unsigned pair_blocks = (n + 11) / 12;  // three particles a warp, four warps a block
+  k_plan<<<grid < 152 ? grid : 152, 256, 0, st>>>(v, x, y, z, radius, n, cohesive ? 1 : 0);
   k_cells<<<grid, 256, 0, st>>>(v, x, y, z, n);
   tds_scan_exclusive(base + kCellCount, base + kCellStart, kMaxCells, base + kTmp, st);
-  e = cudaMemcpyAsync(base + kCursor, base + kCellStart, sizeof(uint32_t) * kMaxCells,
-                      cudaMemcpyDeviceToDevice, st);
-  if (e != cudaSuccess)
-    return tds_set_error_message(TDS_ERR_CUDA, (std::string("tds_find_pair_contacts_noalloc: cudaMemcpyAsync: ") +
-                                                    cudaGetErrorString(e)).c_str());
   k_scatter<<<grid, 256, 0, st>>>(v, n);
-  k_cell_sort<<<kMaxCells / 256, 256, 0, st>>>(v);
-  k_cell_sort_big<<<128, 1024, 0, st>>>(v);
-  k_gather<<<grid, 256, 0, st>>>(v, x, y, z, radius, n);
-  k_pairs<false><<<(n + 127) / 128, 128, 0, st>>>(v, n, nullptr, 0);
+  k_place<<<grid, 256, 0, st>>>(v, x, y, z, radius, n);
+  k_cell_sort_big<<<128, 1024, 0, st>>>(v, x, y, z, radius);
+  k_pairs<false><<<pair_blocks, 128, 0, st>>>(v, n, nullptr, 0, nullptr);
   tds_scan_exclusive(base + kCnt, base + kCStart, n, base + kTmp, st);
-  k_pairs<true><<<(n + 127) / 128, 128, 0, st>>>(v, n, reinterpret_cast<unsigned long long *>(keys), cap);
-  k_total<<<1, 1, 0, st>>>(v, n, count);
+  k_pairs<true><<<pair_blocks, 128, 0, st>>>(v, n, reinterpret_cast<unsigned long long *>(keys), cap, count);
   // the launches above are the only work since the pending-error check on
   // entry, so an error now is theirs
   e = cudaGetLastError();
