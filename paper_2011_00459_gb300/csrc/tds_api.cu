@@ -22,7 +22,7 @@ int tds_launch_features(const DevPtrs &d, const StepConsts &k, int *surf, uint32
 void tds_launch_learned(const DevPtrs &d, const void *packed, uint32_t cap, int compact, cudaStream_t st);
 size_t tds_mlp_packed_bytes();
 int tds_mlp_params();
-void tds_mlp_pack(const float *params, void *packed, cudaStream_t st);
+void tds_mlp_pack(const float *params, void *packed, float *grad, float *loss, cudaStream_t st);
 void tds_mlp_forward_launch(const void *packed, const float *X, uint32_t m, float *Y, cudaStream_t st);
 cudaError_t tds_mlp_loss_grad_launch(const void *packed, const float *X, const float *T, uint32_t m,
                                      float *grad, float *loss, cudaStream_t st);
@@ -1489,7 +1489,7 @@ tds_status tds_set_mlp_weights(tds_scene *s, const float *params, uint32_t count
   if (!s || !params) return fail(TDS_ERR_INVALID_ARG, "NULL argument");
   if ((int)count != tds_mlp_params()) return fail(TDS_ERR_INVALID_ARG, "count must be tds_mlp_param_count()");
   CUDA_TRY(cudaMemcpyAsync(s->x.params, params, sizeof(float) * count, cudaMemcpyHostToDevice, s->st));
-  tds_mlp_pack(s->x.params, s->x.packed, s->st);
+  tds_mlp_pack(s->x.params, s->x.packed, nullptr, nullptr, s->st);
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(s->st));
   s->have_weights = true;
@@ -1534,7 +1534,7 @@ tds_status tds_mlp_forward(const float *params, const float *X, uint32_t m, floa
                            void *stream) {
   if (!params || !X || !Y || !workspace) return fail(TDS_ERR_INVALID_ARG, "NULL argument");
   cudaStream_t st = (cudaStream_t)stream;
-  tds_mlp_pack(params, workspace, st);
+  tds_mlp_pack(params, workspace, nullptr, nullptr, st);
   if (m) tds_mlp_forward_launch(workspace, X, m, Y, st);
   CUDA_TRY(cudaGetLastError());
   return TDS_OK;
@@ -1545,9 +1545,7 @@ tds_status tds_mlp_loss_grad(const float *params, const float *X, const float *T
   if (!params || !X || !T || !grad || !loss || !workspace) return fail(TDS_ERR_INVALID_ARG, "NULL argument");
   if (m == 0) return fail(TDS_ERR_INVALID_ARG, "m must be >= 1");
   cudaStream_t st = (cudaStream_t)stream;
-  CUDA_TRY(cudaMemsetAsync(grad, 0, sizeof(float) * tds_mlp_params(), st));
-  CUDA_TRY(cudaMemsetAsync(loss, 0, sizeof(float), st));
-  tds_mlp_pack(params, workspace, st);
+  tds_mlp_pack(params, workspace, grad, loss, st);
   CUDA_TRY(tds_mlp_loss_grad_launch(workspace, X, T, m, grad, loss, st));
   return TDS_OK;
 }

@@ -44,11 +44,14 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
 }
 
 // Weights as the kernels read them: BF16, K padded to multiples of 16 and the
-// output layer padded to 8 rows; biases FP32.
+// output layer padded to 8 rows; biases FP32. Rows are 8 elements longer than
+// they need be (48 and 144 bytes), so that the eight rows a fragment load
+// touches lie in different banks.
+constexpr int kLdIn = 24, kLdHid = kHid + 8;
 struct Packed {
-  __nv_bfloat16 W1[kHid][16];
-  __nv_bfloat16 W2[kHid][kHid];
-  __nv_bfloat16 W3[8][kHid];
+  __nv_bfloat16 W1[kHid][kLdIn];
+  __nv_bfloat16 W2[kHid][kLdHid];
+  __nv_bfloat16 W3[8][kLdHid];
   float b1[kHid], b2[kHid], b3[8];
 };
 
@@ -121,8 +124,12 @@ __device__ __forceinline__ void forward_tile(const Packed &P, const float *X, ui
   f.y[3] = acc[3] + P.b3[c + 1];
 }
 
-// FP32 master parameters -> packed BF16 weights.
-__global__ void k_pack(const float *params, Packed *P) {
+// FP32 master parameters -> packed BF16 weights; for a training step also the
+// zeros its sums start from (grad and loss, or null).
+__global__ void k_pack(const float *params, Packed *P, float *grad, float *loss) {
+  if (grad)
+    for (int i = threadIdx.x + blockIdx.x * blockDim.x; i < kParams; i += blockDim.x * gridDim.x) grad[i] = 0.f;
+  if (loss && blockIdx.x == 0 && threadIdx.x == 0) *loss = 0.f;
   for (int i = threadIdx.x + blockIdx.x * blockDim.x; i < kHid * 16; i += blockDim.x * gridDim.x) {
     int o = i / 16, k = i % 16;
     P->W1[o][k] = __float2bfloat16_rn(k < kIn ? params[kOffW1 + o * kIn + k] : 0.f);
@@ -166,54 +173,79 @@ __global__ void __launch_bounds__(256) k_forward(const Packed *gP, const float *
 // ---------------------------------------------------------------------------
 constexpr int kTrainWarps = 8;
 constexpr int kRows = 16 * kTrainWarps;  // rows per block iteration
+constexpr int kTiles = 48;               // 16 x 8 tiles of the weight gradients: 8 of dW1, 32 of dW2, 8 of dW3
+constexpr int kWarpTiles = kTiles / kTrainWarps;
+constexpr int kBias = 2 * kHid + 4;      // bias gradients b1, b2, b3
 
-struct Stage {  // per block: the tiles the weight-gradient products read (BF16)
-  __nv_bfloat16 X[kRows][16];
-  __nv_bfloat16 h1[kRows][kHid];
-  __nv_bfloat16 h2[kRows][kHid];
-  __nv_bfloat16 dz1[kRows][kHid];
-  __nv_bfloat16 dz2[kRows][kHid];
-  __nv_bfloat16 dy[kRows][16];
+struct Stage {  // per block: the tiles the weight-gradient products read (BF16, padded rows as Packed's)
+  __nv_bfloat16 X[kRows][kLdIn];
+  __nv_bfloat16 h1[kRows][kLdHid];
+  __nv_bfloat16 h2[kRows][kLdHid];
+  __nv_bfloat16 dz1[kRows][kLdHid];
+  __nv_bfloat16 dz2[kRows][kLdHid];
+  __nv_bfloat16 dy[kRows][kLdIn];
+  float bias[kTrainWarps][kBias];
 };
 
-// A fragment of S^T (S row-major [rows][cols]): A[m][k] = S[k0 + k][m0 + m].
+// Four (two) 8x8 blocks of a row-major matrix, transposed: lane l gives the
+// address of row l mod 8 of block l / 8 and receives, of every block, the
+// elements (2t, g) and (2t + 1, g) (g = l / 4, t = l mod 4).
+__device__ __forceinline__ void ldsm_t4(const void *row, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(row)))
+               : "memory");
+}
+__device__ __forceinline__ void ldsm_t2(const void *row, uint32_t &r0, uint32_t &r1) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+               : "=r"(r0), "=r"(r1)
+               : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(row)))
+               : "memory");
+}
+// A fragment of S^T (S row-major [rows][cols]): A[m][k] = S[k0 + k][m0 + m];
+// its registers are the blocks (k 0, m 0), (k 0, m 8), (k 8, m 0), (k 8, m 8).
 template <int C>
 __device__ __forceinline__ void frag_at(const __nv_bfloat16 (*S)[C], int k0, int m0, uint32_t (&a)[4]) {
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  a[0] = pack_raw(S[k0 + 2 * t][m0 + g], S[k0 + 2 * t + 1][m0 + g]);
-  a[1] = pack_raw(S[k0 + 2 * t][m0 + g + 8], S[k0 + 2 * t + 1][m0 + g + 8]);
-  a[2] = pack_raw(S[k0 + 2 * t + 8][m0 + g], S[k0 + 2 * t + 9][m0 + g]);
-  a[3] = pack_raw(S[k0 + 2 * t + 8][m0 + g + 8], S[k0 + 2 * t + 9][m0 + g + 8]);
+  const int lane = threadIdx.x & 31;
+  ldsm_t4(&S[k0 + (lane & 7) + (lane & 16 ? 8 : 0)][m0 + (lane & 8)], a);
 }
-// B fragment of S itself (B[k][n] = S[k0 + k][n0 + n]).
+// B fragment of S itself (B[k][n] = S[k0 + k][n0 + n]): blocks (k 0), (k 8).
 template <int C>
 __device__ __forceinline__ void frag_b(const __nv_bfloat16 (*S)[C], int k0, int n0, uint32_t &b0, uint32_t &b1) {
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  b0 = pack_raw(S[k0 + 2 * t][n0 + g], S[k0 + 2 * t + 1][n0 + g]);
-  b1 = pack_raw(S[k0 + 2 * t + 8][n0 + g], S[k0 + 2 * t + 9][n0 + g]);
+  const int lane = threadIdx.x & 31;
+  ldsm_t2(&S[k0 + (lane & 15)][n0], b0, b1);
 }
 
 // Sum over the 8 lanes sharing t (the 16 rows) of a per-column value; lane t
-// (< 4) adds it to dst when valid.
+// (< 4) adds it to dst (its warp's own) when valid.
 __device__ __forceinline__ void col_sum_add(float v, float *dst, bool valid = true) {
   v += __shfl_xor_sync(0xffffffffu, v, 4);
   v += __shfl_xor_sync(0xffffffffu, v, 8);
   v += __shfl_xor_sync(0xffffffffu, v, 16);
-  if ((threadIdx.x & 31) < 4 && valid) atomicAdd(dst, v);
+  if ((threadIdx.x & 31) < 4 && valid) *dst += v;
 }
 
+// What bounds it: latency (a minibatch of 8192 rows is one pass of 64 blocks).
+// Fragments come by ldmatrix from padded rows, the weight gradients stay in the
+// tensor-core accumulators over all of a block's rows and the bias gradients in
+// shared memory, so that a block ends with one addition per parameter. 8192
+// rows: 11.7 us; with 2-byte fragment loads, 8-way bank conflicts and every
+// 128 rows' sums added to global memory 26.1.
 __global__ void __launch_bounds__(kTrainWarps * 32) k_loss_grad(const Packed *gP, const float *X,
                                                                  const float *T, uint32_t m,
                                                                  float *grad, float *loss) {
-  __shared__ Packed P;
+  __shared__ __align__(16) Packed P;
   extern __shared__ __align__(16) unsigned char dyn[];
   Stage &S = *reinterpret_cast<Stage *>(dyn);
   for (int i = threadIdx.x; i < (int)(sizeof(Packed) / 4); i += blockDim.x)
     reinterpret_cast<uint32_t *>(&P)[i] = reinterpret_cast<const uint32_t *>(gP)[i];
+  for (int i = threadIdx.x; i < kTrainWarps * kBias; i += blockDim.x) (&S.bias[0][0])[i] = 0.f;
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const float scale = 2.0f / (3.0f * (float)m);
+  float *bias = S.bias[warp];
   float lsum = 0.f;
+  float wacc[kWarpTiles][4] = {};  // this warp's tiles of the weight gradients
   for (uint32_t base = blockIdx.x * kRows; base < m; base += gridDim.x * kRows) {
     const uint32_t row0 = base + warp * 16;
     const int r0 = warp * 16;  // this warp's rows in the stage
@@ -230,18 +262,23 @@ __global__ void __launch_bounds__(kTrainWarps * 32) k_loss_grad(const Packed *gP
       lsum += e * e;
       dy[q] = scale * e;
     }
-    col_sum_add(dy[0] + dy[2], &grad[kOffB3 + min(2 * t, kOut - 1)], 2 * t < kOut);
-    col_sum_add(dy[1] + dy[3], &grad[kOffB3 + min(2 * t + 1, kOut - 1)], 2 * t + 1 < kOut);
+    col_sum_add(dy[0] + dy[2], bias + 2 * kHid + min(2 * t, kOut - 1), 2 * t < kOut);
+    col_sum_add(dy[1] + dy[3], bias + 2 * kHid + min(2 * t + 1, kOut - 1), 2 * t + 1 < kOut);
     // dh2 = dy W3 (K = 8 outputs, padded to 16)
     uint32_t Ady[4] = {pack_bf16(dy[0], dy[1]), pack_bf16(dy[2], dy[3]), 0u, 0u};
     float dz2[8][4];
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      uint32_t b0 = pack_raw(P.W3[2 * t][nt * 8 + g], P.W3[2 * t + 1][nt * 8 + g]);
-      mma16816(acc, Ady, b0, 0u);
+    for (int np = 0; np < 4; ++np) {  // pairs of column tiles: one fragment load of two 8x8 blocks
+      uint32_t b0, b1;
+      ldsm_t2(&P.W3[lane & 7][np * 16 + (lane & 8)], b0, b1);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) dz2[nt][q] = f.z2[nt][q] > 0.f ? acc[q] : 0.f;
+      for (int h = 0; h < 2; ++h) {
+        const int nt = 2 * np + h;
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        mma16816(acc, Ady, h ? b1 : b0, 0u);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dz2[nt][q] = f.z2[nt][q] > 0.f ? acc[q] : 0.f;
+      }
     }
     // dh1 = dz2 W2
     uint32_t Adz2[4][4];
@@ -257,10 +294,11 @@ __global__ void __launch_bounds__(kTrainWarps * 32) k_loss_grad(const Packed *gP
     for (int nt = 0; nt < 8; ++nt) {
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int kc = 0; kc < 4; ++kc) {
-        uint32_t b0 = pack_raw(P.W2[kc * 16 + 2 * t][nt * 8 + g], P.W2[kc * 16 + 2 * t + 1][nt * 8 + g]);
-        uint32_t b1 = pack_raw(P.W2[kc * 16 + 2 * t + 8][nt * 8 + g], P.W2[kc * 16 + 2 * t + 9][nt * 8 + g]);
-        mma16816(acc, Adz2[kc], b0, b1);
+      for (int kc = 0; kc < 4; kc += 2) {
+        uint32_t b[4];  // (k 0, k 8) of chunk kc, then of kc + 1
+        ldsm_t4(&P.W2[kc * 16 + lane][nt * 8], b);
+        mma16816(acc, Adz2[kc], b[0], b[1]);
+        mma16816(acc, Adz2[kc + 1], b[2], b[3]);
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) dz1[nt][q] = f.z1[nt][q] > 0.f ? acc[q] : 0.f;
@@ -269,10 +307,10 @@ __global__ void __launch_bounds__(kTrainWarps * 32) k_loss_grad(const Packed *gP
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
       const int c = nt * 8 + 2 * t;
-      col_sum_add(dz2[nt][0] + dz2[nt][2], &grad[kOffB2 + c]);
-      col_sum_add(dz2[nt][1] + dz2[nt][3], &grad[kOffB2 + c + 1]);
-      col_sum_add(dz1[nt][0] + dz1[nt][2], &grad[kOffB1 + c]);
-      col_sum_add(dz1[nt][1] + dz1[nt][3], &grad[kOffB1 + c + 1]);
+      col_sum_add(dz2[nt][0] + dz2[nt][2], bias + kHid + c);
+      col_sum_add(dz2[nt][1] + dz2[nt][3], bias + kHid + c + 1);
+      col_sum_add(dz1[nt][0] + dz1[nt][2], bias + c);
+      col_sum_add(dz1[nt][1] + dz1[nt][3], bias + c + 1);
     }
     // stage the tiles the weight gradients read
     for (int k = lane; k < 16 * 16; k += 32) {
@@ -283,44 +321,57 @@ __global__ void __launch_bounds__(kTrainWarps * 32) k_loss_grad(const Packed *gP
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int r = r0 + g + (q >> 1) * 8, c = nt * 8 + 2 * t + (q & 1);
-        S.h1[r][c] = __float2bfloat16_rn(fmaxf(f.z1[nt][q], 0.f));
-        S.h2[r][c] = __float2bfloat16_rn(fmaxf(f.z2[nt][q], 0.f));
-        S.dz1[r][c] = __float2bfloat16_rn(dz1[nt][q]);
-        S.dz2[r][c] = __float2bfloat16_rn(dz2[nt][q]);
+      for (int q = 0; q < 4; q += 2) {
+        const int r = r0 + g + (q >> 1) * 8, c = nt * 8 + 2 * t;
+        *reinterpret_cast<uint32_t *>(&S.h1[r][c]) = pack_bf16(fmaxf(f.z1[nt][q], 0.f), fmaxf(f.z1[nt][q + 1], 0.f));
+        *reinterpret_cast<uint32_t *>(&S.h2[r][c]) = pack_bf16(fmaxf(f.z2[nt][q], 0.f), fmaxf(f.z2[nt][q + 1], 0.f));
+        *reinterpret_cast<uint32_t *>(&S.dz1[r][c]) = pack_bf16(dz1[nt][q], dz1[nt][q + 1]);
+        *reinterpret_cast<uint32_t *>(&S.dz2[r][c]) = pack_bf16(dz2[nt][q], dz2[nt][q + 1]);
       }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = r0 + g + (q >> 1) * 8, c = 2 * t + (q & 1);
-      S.dy[r][c] = __float2bfloat16_rn(dy[q]);
-      S.dy[r][c + 8] = __float2bfloat16_rn(0.f);
+    for (int q = 0; q < 4; q += 2) {
+      const int r = r0 + g + (q >> 1) * 8, c = 2 * t;
+      *reinterpret_cast<uint32_t *>(&S.dy[r][c]) = pack_bf16(dy[q], dy[q + 1]);
+      *reinterpret_cast<uint32_t *>(&S.dy[r][c + 8]) = 0u;
     }
     __syncthreads();
     // weight gradients over the block's kRows rows: 8 tiles of dW1 (64x16),
     // 32 of dW2 (64x64), 8 of dW3 (8x64, M padded to 16)
-    for (int tile = warp; tile < 48; tile += kTrainWarps) {
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      int which, mt, nt;
-      if (tile < 8) { which = 1; mt = tile >> 1; nt = tile & 1; }
-      else if (tile < 40) { which = 2; mt = (tile - 8) >> 3; nt = (tile - 8) & 7; }
-      else { which = 3; mt = 0; nt = tile - 40; }
+#pragma unroll
+    for (int w = 0; w < kWarpTiles; ++w) {
+      const int tile = warp + w * kTrainWarps;
+#pragma unroll
       for (int kc = 0; kc < kRows / 16; ++kc) {
         uint32_t a[4], b0, b1;
-        if (which == 1) { frag_at<kHid>(S.dz1, kc * 16, mt * 16, a); frag_b<16>(S.X, kc * 16, nt * 8, b0, b1); }
-        else if (which == 2) { frag_at<kHid>(S.dz2, kc * 16, mt * 16, a); frag_b<kHid>(S.h1, kc * 16, nt * 8, b0, b1); }
-        else { frag_at<16>(S.dy, kc * 16, 0, a); frag_b<kHid>(S.h2, kc * 16, nt * 8, b0, b1); }
-        mma16816(acc, a, b0, b1);
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int o = mt * 16 + g + (q >> 1) * 8, i = nt * 8 + 2 * t + (q & 1);
-        if (which == 1) { if (i < kIn) atomicAdd(&grad[kOffW1 + o * kIn + i], acc[q]); }
-        else if (which == 2) atomicAdd(&grad[kOffW2 + o * kHid + i], acc[q]);
-        else if (o < kOut) atomicAdd(&grad[kOffW3 + o * kHid + i], acc[q]);
+        if (tile < 8) { frag_at(S.dz1, kc * 16, (tile >> 1) * 16, a); frag_b(S.X, kc * 16, (tile & 1) * 8, b0, b1); }
+        else if (tile < 40) { frag_at(S.dz2, kc * 16, ((tile - 8) >> 3) * 16, a); frag_b(S.h1, kc * 16, ((tile - 8) & 7) * 8, b0, b1); }
+        else { frag_at(S.dy, kc * 16, 0, a); frag_b(S.h2, kc * 16, (tile - 40) * 8, b0, b1); }
+        mma16816(wacc[w], a, b0, b1);
       }
     }
     __syncthreads();
+  }
+  // one addition per parameter and block
+#pragma unroll
+  for (int w = 0; w < kWarpTiles; ++w) {
+    const int tile = warp + w * kTrainWarps;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int o = g + (q >> 1) * 8, i = 2 * t + (q & 1);
+      if (tile < 8) {
+        if ((tile & 1) * 8 + i < kIn) atomicAdd(&grad[kOffW1 + ((tile >> 1) * 16 + o) * kIn + (tile & 1) * 8 + i], wacc[w][q]);
+      } else if (tile < 40) {
+        atomicAdd(&grad[kOffW2 + (((tile - 8) >> 3) * 16 + o) * kHid + ((tile - 8) & 7) * 8 + i], wacc[w][q]);
+      } else if (o < kOut) {
+        atomicAdd(&grad[kOffW3 + o * kHid + (tile - 40) * 8 + i], wacc[w][q]);
+      }
+    }
+  }
+  __syncthreads();  // (a block without rows has not passed one since it cleared the bias sums)
+  for (int c = threadIdx.x; c < 2 * kHid + kOut; c += blockDim.x) {
+    float v = 0.f;
+    for (int w = 0; w < kTrainWarps; ++w) v += S.bias[w][c];
+    atomicAdd(&grad[c < kHid ? kOffB1 + c : (c < 2 * kHid ? kOffB2 + c - kHid : kOffB3 + c - 2 * kHid)], v);
   }
   // loss
   lsum += __shfl_xor_sync(0xffffffffu, lsum, 1);
@@ -535,8 +586,8 @@ void tds_launch_learned(const DevPtrs &d, const void *packed, uint32_t cap, int 
 size_t tds_mlp_packed_bytes() { return (sizeof(Packed) + 255) & ~(size_t)255; }
 int tds_mlp_params() { return kParams; }
 
-void tds_mlp_pack(const float *params, void *packed, cudaStream_t st) {
-  k_pack<<<8, 256, 0, st>>>(params, static_cast<Packed *>(packed));
+void tds_mlp_pack(const float *params, void *packed, float *grad, float *loss, cudaStream_t st) {
+  k_pack<<<24, 256, 0, st>>>(params, static_cast<Packed *>(packed), grad, loss);
 }
 void tds_mlp_forward_launch(const void *packed, const float *X, uint32_t m, float *Y, cudaStream_t st) {
   unsigned blocks = (m + 16 * 8 - 1) / (16 * 8);
