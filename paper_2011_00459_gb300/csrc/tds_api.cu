@@ -382,7 +382,6 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
   d.cell_of = c.take<uint32_t>(n);
   d.cell_count = c.take<uint32_t>(L.ncells + 2);  // + the trailing cell of dormant slots
   d.cell_start = c.take<uint32_t>(L.ncells + 2);
-  d.cell_cursor = c.take<uint32_t>(L.ncells + 1);
   d.perm = c.take<uint32_t>(n);
   d.cnt = c.take<uint32_t>(n + 1);
   d.cstart = c.take<uint32_t>(n + 1);
@@ -393,7 +392,7 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
   d.c_sv = c.take<float4>(cap); d.c_sw = c.take<float4>(cap);
   d.c_la = c.take<float4>(cap); d.c_lb = c.take<float2>(cap);
   d.inc_cnt = c.take<uint32_t>(n + 1); d.inc_start = c.take<uint32_t>(n + 1);
-  d.inc_cursor = c.take<uint32_t>(n); d.inc_ent = c.take<uint2>(2 * (size_t)cap);
+  d.inc_ent = c.take<uint2>(2 * (size_t)cap);
   d.prio = c.take<unsigned long long>(cap);
   d.colour = c.take<uint8_t>(cap);
   d.cmask = c.take<ulonglong2>(n);
@@ -691,7 +690,10 @@ tds_status create_impl(const tds_scene_desc *descs, uint32_t count, void *worksp
   s->sms = sms;
   // the default solver shape's co-resident CTAs at most
   s->pgs_blocks = pgs_blocks_for(s->L.n, sms * std::max(1, tds_pgs_occupancy(0)));
-  s->colour_blocks = sms * (occ_col < 4 ? occ_col : 4);
+  // a thread per contact or so (3 to 4 a particle): more blocks only wait at
+  // the rounds' barriers
+  s->colour_blocks = std::max(1, (int)std::min<uint64_t>((uint64_t)sms * (occ_col < 4 ? occ_col : 4),
+                                                         ((uint64_t)s->L.n * 4 + 255) / 256));
   s->max_pgs_blocks = 64 * sms;  // the workspace's limit; each shape's co-residency limits it further
   s->max_colour_blocks = sms * occ_col;
   Carver probe{nullptr};

@@ -16,26 +16,16 @@ namespace {
 
 __device__ __forceinline__ bool is_dyn(uint32_t b) { return (b & TDS_STATIC) == 0u; }
 
-// Incidence counts per particle (the priorities were written with the
-// contacts).
-__global__ void k_inc_count(DevPtrs d) {
-  const uint32_t nc = d.ctr[CTR_NC];
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
-    uint2 ab = d.c_ab[c];
-    atomicAdd(d.inc_cnt + ab.x, 1u);
-    if (is_dyn(ab.y)) atomicAdd(d.inc_cnt + ab.y, 1u);
-  }
-}
-
 // Incidence entries carry the contact id and the high word of its priority,
-// so walking a neighbourhood needs no dependent loads to compare priorities.
+// so walking a neighbourhood needs no dependent loads to compare priorities
+// (counted, with each contact's place, when the rows were written).
 __global__ void k_inc_fill(DevPtrs d) {
   const uint32_t nc = d.ctr[CTR_NC];
   for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
     uint2 ab = d.c_ab[c];
     uint32_t hi = (uint32_t)(d.prio[c] >> 32);
-    d.inc_ent[atomicAdd(d.inc_cursor + ab.x, 1u)] = make_uint2(c, hi);
-    if (is_dyn(ab.y)) d.inc_ent[atomicAdd(d.inc_cursor + ab.y, 1u)] = make_uint2(c, hi);
+    d.inc_ent[d.inc_start[ab.x] + d.frontier0[c]] = make_uint2(c, hi);
+    if (is_dyn(ab.y)) d.inc_ent[d.inc_start[ab.y] + d.frontier1[c]] = make_uint2(c, hi);
   }
 }
 
@@ -235,72 +225,161 @@ __device__ __forceinline__ uint32_t bucket_of(const DevPtrs &d, uint32_t c) {
   return 2u * col + (is_dyn(d.c_ab[c].y) ? 0u : 1u);
 }
 
-__global__ void k_bucket_hist(DevPtrs d) {
+// Only the buckets and tiles in use are counted and scanned: the histogram is
+// (buckets 0 .. 2 colours) x (tiles of the contacts there are), its length in
+// CTR_HIST (all 256 buckets of the whole capacity are 50 times that).
+constexpr int kBucketThreads = 1024;
+
+__device__ __forceinline__ uint32_t used_buckets(const DevPtrs &d) {
+  return 2u * min(d.ctr[CTR_NCOL], (uint32_t)TDS_MAX_COLOURS);
+}
+__device__ __forceinline__ uint32_t used_tiles(uint32_t nc) { return (nc + TDS_TILE - 1u) / TDS_TILE; }
+
+__global__ void __launch_bounds__(kBucketThreads) k_bucket_hist(DevPtrs d) {
   __shared__ uint32_t hist[TDS_NBUCKETS];
-  const uint32_t nc = d.ctr[CTR_NC];
+  const uint32_t nc = d.ctr[CTR_NC], nt = used_tiles(nc), nb = used_buckets(d);
+  if (blockIdx.x == 0 && threadIdx.x == 0) d.ctr[CTR_HIST] = nb * nt;
+  if (blockIdx.x >= nt) return;
   for (uint32_t b = threadIdx.x; b < TDS_NBUCKETS; b += blockDim.x) hist[b] = 0;
   __syncthreads();
-  uint32_t base = blockIdx.x * TDS_TILE;
+  const uint32_t base = blockIdx.x * TDS_TILE, lane = threadIdx.x & 31u;
   for (uint32_t k = threadIdx.x; k < TDS_TILE; k += blockDim.x) {
-    uint32_t c = base + k;
+    const uint32_t c = base + k;
+    uint32_t bk = 0xFFFFFFFFu;
     if (c < nc) {
       if (d.colour[c] >= TDS_MAX_COLOURS) latch_error(d.err, DEV_ERR_CAPACITY);
-      atomicAdd(hist + bucket_of(d, c), 1u);
+      bk = bucket_of(d, c);
     }
+    const uint32_t peers = __match_any_sync(0xffffffffu, bk);  // one addition per bucket and warp
+    if (bk != 0xFFFFFFFFu && (peers & ((1u << lane) - 1u)) == 0u) atomicAdd(hist + bk, (uint32_t)__popc(peers));
   }
   __syncthreads();
-  for (uint32_t b = threadIdx.x; b < TDS_NBUCKETS; b += blockDim.x)
-    d.tile_hist[b * d.ntiles + blockIdx.x] = hist[b];
+  for (uint32_t b = threadIdx.x; b < nb; b += blockDim.x) d.tile_hist[b * nt + blockIdx.x] = hist[b];
+}
+
+// Exclusive prefix sum of one value per thread over a block of T threads;
+// *total receives the sum.
+template <int T>
+__device__ __forceinline__ uint32_t block_prefix(uint32_t v, uint32_t *total) {
+  __shared__ uint32_t sums[T / 32 + 1];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  uint32_t inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t up = __shfl_up_sync(0xffffffffu, inc, o);
+    if ((int)lane >= o) inc += up;
+  }
+  if (lane == 31u) sums[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t s = lane < T / 32 ? sums[lane] : 0u;
+    uint32_t si = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t up = __shfl_up_sync(0xffffffffu, si, o);
+      if ((int)lane >= o) si += up;
+    }
+    if (lane < T / 32) sums[lane] = si - s;
+    if (lane == T / 32 - 1) sums[T / 32] = si;
+  }
+  __syncthreads();
+  const uint32_t r = inc - v + sums[warp];
+  *total = sums[T / 32];
+  __syncthreads();
+  return r;
+}
+
+// Residual chunks. Inside a bucket the contacts keep the owner order, which
+// is scene-major (slots are sorted by cell, cells by scene), so each scene's
+// contacts of a bucket form one range; its start is the bucket's start plus
+// the contacts of the earlier scenes. Each range is cut into chunks of at
+// most TDS_RES_CHUNK contacts, numbered scene-major (scene, bucket, piece):
+// a scene's chunks are consecutive, and they are the same chunks whether the
+// scene is stepped alone or in a batch.
+__device__ __forceinline__ uint32_t pieces(uint32_t cnt) { return (cnt + TDS_RES_CHUNK - 1u) / TDS_RES_CHUNK; }
+// (thread t of n writes every n-th of them)
+__device__ __forceinline__ void write_chunks(const DevPtrs &d, uint32_t first, uint32_t start, uint32_t cnt, uint32_t q,
+                                             uint32_t t, uint32_t n) {
+  for (uint32_t k = t; k * TDS_RES_CHUNK < cnt; k += n)
+    d.chunk[first + k] = make_uint4(start + k * TDS_RES_CHUNK, min(TDS_RES_CHUNK, cnt - k * TDS_RES_CHUNK), q, 0u);
 }
 
 // Bucket ranges in the padded colour order: every bucket starts at a multiple
-// of 4 contacts (16-byte aligned rows for bulk copies); padding slots carry
-// order == 0xFFFFFFFF and are never solved.
-__global__ void k_bucket_starts(DevPtrs d) {
-  if (threadIdx.x != 0) return;
-  uint32_t run = 0;
-  for (uint32_t b = 0; b < TDS_NBUCKETS; ++b) {
-    uint32_t u0 = d.tile_off[b * d.ntiles];
-    uint32_t u1 = b + 1 < TDS_NBUCKETS ? d.tile_off[(b + 1) * d.ntiles] : d.ctr[CTR_NC];
-    uint32_t cnt = u1 - u0;
-    d.bstart[b] = run;
-    d.bend[b] = run + cnt;
-    d.bpad[b] = run - u0;
-    run += (cnt + 3u) & ~3u;
+// of 4 contacts (16-byte aligned rows); padding slots carry
+// order == 0xFFFFFFFF and are never solved. For a single scene also its
+// residual chunks. One block, a thread per bucket (one thread for all of them:
+// 110 us against 4).
+__global__ void __launch_bounds__(TDS_NBUCKETS) k_bucket_starts(DevPtrs d) {
+  const uint32_t nc = d.ctr[CTR_NC], nt = used_tiles(nc), nb = used_buckets(d), b = threadIdx.x;
+  const uint32_t u0 = b < nb && nt ? d.tile_off[b * nt] : nc, u1 = b + 1u < nb && nt ? d.tile_off[(b + 1u) * nt] : nc;
+  const uint32_t cnt = u1 - u0, padded = (cnt + 3u) & ~3u;
+  uint32_t total;
+  const uint32_t start = block_prefix<TDS_NBUCKETS>(padded, &total);
+  d.bstart[b] = start;
+  d.bend[b] = start + cnt;
+  d.bpad[b] = start - u0;
+  for (uint32_t p = start + cnt; p < start + padded; ++p) d.order[p] = 0xFFFFFFFFu;
+  if (b == 0u) {
+    d.bstart[TDS_NBUCKETS] = total;
+    d.ctr[CTR_PADDED] = total;
   }
-  d.bstart[TDS_NBUCKETS] = run;
-  d.ctr[CTR_PADDED] = run;
+  if (d.nscenes == 1u) {
+    d.scq_cnt[b] = cnt;
+    uint32_t nchunk;
+    const uint32_t first = block_prefix<TDS_NBUCKETS>(pieces(cnt), &nchunk);
+    __shared__ uint32_t s_first[TDS_NBUCKETS], s_start[TDS_NBUCKETS], s_cnt[TDS_NBUCKETS];
+    s_first[b] = first;
+    s_start[b] = start;
+    s_cnt[b] = cnt;
+    d.scq_chunk[b] = first;
+    if (b == 0u) {
+      d.scq_chunk[TDS_NBUCKETS] = nchunk;
+      d.ctr[CTR_NCHUNK] = nchunk;
+    }
+    __syncthreads();
+    for (uint32_t g = 0; g < nb; ++g) write_chunks(d, s_first[g], s_start[g], s_cnt[g], 0u, b, TDS_NBUCKETS);
+  }
 }
 
 // Scatter every contact's rows to its colour-order position: tile offset of
 // its bucket + rank among equal buckets earlier in the tile (warp match +
 // per-warp counts), so the order inside a bucket is the owner order.
-__global__ void __launch_bounds__(256) k_bucket_scatter(DevPtrs d) {
-  constexpr int W = 8;  // warps per block
+__global__ void __launch_bounds__(kBucketThreads) k_bucket_scatter(DevPtrs d) {
+  constexpr uint32_t W = kBucketThreads / 32;  // warps per block
   __shared__ uint32_t base[TDS_NBUCKETS];
-  __shared__ uint32_t wcnt[W][TDS_NBUCKETS];
-  const uint32_t nc = d.ctr[CTR_NC];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (uint32_t b = threadIdx.x; b < TDS_NBUCKETS; b += blockDim.x)
-    base[b] = d.tile_off[b * d.ntiles + blockIdx.x];
-  for (uint32_t chunk = 0; chunk < TDS_TILE; chunk += 256) {
-    for (uint32_t q = threadIdx.x; q < W * TDS_NBUCKETS; q += blockDim.x) (&wcnt[0][0])[q] = 0;
-    __syncthreads();
-    uint32_t c = blockIdx.x * TDS_TILE + chunk + threadIdx.x;
-    bool live = c < nc;
-    uint32_t bk = live ? bucket_of(d, c) : 0xFFFFFFFFu;
-    uint32_t peers = __match_any_sync(0xffffffffu, bk);
-    uint32_t rank_in_warp = __popc(peers & ((1u << lane) - 1u));
+  __shared__ uint32_t wcnt[W][TDS_NBUCKETS + 1];
+  const uint32_t nc = d.ctr[CTR_NC], nt = used_tiles(nc), nb = used_buckets(d);
+  if (blockIdx.x >= nt) return;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  for (uint32_t b = threadIdx.x; b < nb; b += blockDim.x) base[b] = d.tile_off[b * nt + blockIdx.x] + d.bpad[b];
+  for (uint32_t chunk = 0; chunk < TDS_TILE; chunk += kBucketThreads) {
+    for (uint32_t b = lane; b < nb; b += 32u) wcnt[warp][b] = 0;
+    __syncwarp();
+    const uint32_t c = blockIdx.x * TDS_TILE + chunk + threadIdx.x;
+    uint32_t bk = c < nc ? bucket_of(d, c) : 0xFFFFFFFFu;
+    const bool live = bk < nb;  // (a colouring that gave up leaves contacts outside the counted buckets: the step has failed)
+    if (!live) bk = 0xFFFFFFFFu;
+    const uint32_t peers = __match_any_sync(0xffffffffu, bk);
+    const uint32_t rank_in_warp = __popc(peers & ((1u << lane) - 1u));
     if (live && rank_in_warp == 0) wcnt[warp][bk] = __popc(peers);
     __syncthreads();
-    for (uint32_t b = threadIdx.x; b < TDS_NBUCKETS; b += blockDim.x) {
-      uint32_t run = base[b];
-      for (int w = 0; w < W; ++w) { uint32_t t = wcnt[w][b]; wcnt[w][b] = run; run += t; }
-      base[b] = run;
+    // per bucket, the warps' places: a warp per bucket, a lane per warp of the block
+    for (uint32_t b = warp; b < nb; b += W) {
+      const uint32_t v = wcnt[lane][b];
+      uint32_t inc = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t up = __shfl_up_sync(0xffffffffu, inc, o);
+        if ((int)lane >= o) inc += up;
+      }
+      const uint32_t at = base[b];
+      wcnt[lane][b] = at + inc - v;
+      __syncwarp();
+      if (lane == 31u) base[b] = at + inc;
     }
     __syncthreads();
     if (live) {
-      uint32_t p = wcnt[warp][bk] + rank_in_warp + d.bpad[bk];
+      const uint32_t p = wcnt[warp][bk] + rank_in_warp;
       const uint2 ab = d.c_ab[c];
       d.order[p] = c;
       d.p_ab[p] = ab;
@@ -319,60 +398,57 @@ __global__ void __launch_bounds__(256) k_bucket_scatter(DevPtrs d) {
       if (bk & 1u) { d.p_sv[p] = d.c_sv[c]; d.p_sw[p] = d.c_sw[c]; }
       d.p_la[p] = d.c_la[c];
       d.p_lb[p] = d.c_lb[c];
-      if (d.nscenes > 1) atomicAdd(d.scq_cnt + (size_t)d.sid[ab.x] * TDS_NBUCKETS + bk, 1u);
+    }
+    if (d.nscenes > 1) {  // contacts per (scene, bucket); a warp's contacts are nearly always one scene's
+      const uint32_t q = live ? d.sid[d.c_ab[c].x] : 0xFFFFFFFFu;
+      const uint32_t same = __match_any_sync(0xffffffffu, q) & peers;
+      if (live && (same & ((1u << lane) - 1u)) == 0u)
+        atomicAdd(d.scq_cnt + (size_t)q * TDS_NBUCKETS + bk, (uint32_t)__popc(same));
     }
     __syncthreads();
   }
 }
 
-// Residual chunks. Inside a bucket the contacts keep the owner order, which
-// is scene-major (slots are sorted by cell, cells by scene), so each scene's
-// contacts of a bucket form one range; its start is the bucket's start plus
-// the contacts of the earlier scenes. Each range is cut into chunks of at
-// most TDS_RES_CHUNK contacts, numbered scene-major (scene, bucket, piece):
-// a scene's chunks are consecutive, and they are the same chunks whether the
-// scene is stepped alone or in a batch. One block.
+// The residual chunks of a batch, over its scenes and the buckets in use. One block.
 __global__ void __launch_bounds__(1024) k_scene_chunks(DevPtrs d) {
   constexpr uint32_t NB = TDS_NBUCKETS;
-  const uint32_t S = d.nscenes, total = S * NB;
-  __shared__ uint32_t part[1024];
-  for (uint32_t b = threadIdx.x; b < NB; b += blockDim.x) {
+  const uint32_t S = d.nscenes, nb = used_buckets(d), lane = threadIdx.x & 31u;
+  // a warp per bucket: the scenes' starts in it
+  for (uint32_t b = threadIdx.x >> 5; b < nb; b += 32u) {
     uint32_t run = d.bstart[b];
-    for (uint32_t q = 0; q < S; ++q) {
-      const size_t e = (size_t)q * NB + b;
-      const uint32_t cnt = S == 1 ? d.bend[b] - d.bstart[b] : d.scq_cnt[e];
-      if (S == 1) d.scq_cnt[e] = cnt;
-      d.scq_start[e] = run;
-      run += cnt;
+    for (uint32_t q0 = 0; q0 < S; q0 += 32u) {
+      const uint32_t q = q0 + lane;
+      const uint32_t v = q < S ? d.scq_cnt[(size_t)q * NB + b] : 0u;
+      uint32_t inc = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t up = __shfl_up_sync(0xffffffffu, inc, o);
+        if ((int)lane >= o) inc += up;
+      }
+      if (q < S) d.scq_start[(size_t)q * NB + b] = run + inc - v;
+      run += __shfl_sync(0xffffffffu, inc, 31);
     }
   }
   __syncthreads();
-  // exclusive scan of the pieces over (scene, bucket): each thread a
-  // contiguous segment, then a scan of the segment sums
-  const uint32_t seg = (total + blockDim.x - 1) / blockDim.x;
-  const uint32_t lo = min(threadIdx.x * seg, total), hi = min(lo + seg, total);
-  uint32_t sum = 0;
-  for (uint32_t e = lo; e < hi; ++e) sum += (d.scq_cnt[e] + TDS_RES_CHUNK - 1u) / TDS_RES_CHUNK;
-  part[threadIdx.x] = sum;
-  __syncthreads();
+  // number the pieces scene-major
+  uint32_t carry = 0;
+  for (uint32_t e0 = 0; e0 < S * nb; e0 += blockDim.x) {
+    const uint32_t e = e0 + threadIdx.x, q = e / max(nb, 1u), b = e - q * nb;
+    const size_t at = (size_t)q * NB + b;
+    const uint32_t cnt = e < S * nb ? d.scq_cnt[at] : 0u;
+    uint32_t total;
+    const uint32_t first = carry + block_prefix<1024>(pieces(cnt), &total);
+    if (e < S * nb) {
+      if (b == 0u) d.scq_chunk[at] = first;  // (only the scenes' first chunks are asked for)
+      write_chunks(d, first, d.scq_start[at], cnt, q, 0u, 1u);
+    }
+    carry += total;
+  }
+  if (nb == 0u)
+    for (uint32_t q = threadIdx.x; q < S; q += blockDim.x) d.scq_chunk[(size_t)q * NB] = 0u;
   if (threadIdx.x == 0) {
-    uint32_t run = 0;
-    for (uint32_t t = 0; t < blockDim.x; ++t) {
-      const uint32_t v = part[t];
-      part[t] = run;
-      run += v;
-    }
-    d.scq_chunk[total] = run;
-    d.ctr[CTR_NCHUNK] = run;
-  }
-  __syncthreads();
-  uint32_t base = part[threadIdx.x];
-  for (uint32_t e = lo; e < hi; ++e) {
-    d.scq_chunk[e] = base;
-    const uint32_t cnt = d.scq_cnt[e], start = d.scq_start[e], q = e / NB;
-    for (uint32_t k = 0; k * TDS_RES_CHUNK < cnt; ++k)
-      d.chunk[base + k] = make_uint4(start + k * TDS_RES_CHUNK, min(TDS_RES_CHUNK, cnt - k * TDS_RES_CHUNK), q, 0u);
-    base += (cnt + TDS_RES_CHUNK - 1u) / TDS_RES_CHUNK;
+    d.scq_chunk[(size_t)S * NB] = carry;
+    d.ctr[CTR_NCHUNK] = carry;
   }
 }
 
@@ -384,10 +460,7 @@ int tds_launch_colouring(const DevPtrs &d, uint32_t n, uint32_t cap, int coop_bl
   unsigned gc = (cap + 255) / 256;
   if (gc > 152 * 16) gc = 152 * 16;
   if (gc == 0) gc = 1;
-  cudaMemsetAsync(d.inc_cnt, 0, sizeof(uint32_t) * (n + 1), st);
-  k_inc_count<<<gc, 256, 0, st>>>(d);
   scans += tds_scan_exclusive(d.inc_cnt, d.inc_start, n, d.scan_tmp, st);
-  cudaMemcpyAsync(d.inc_cursor, d.inc_start, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st);
   k_inc_fill<<<gc, 256, 0, st>>>(d);
   cudaMemsetAsync(d.ctr + CTR_FCOUNT, 0, 3 * sizeof(uint32_t), st);
   cudaMemsetAsync(d.ctr + CTR_NCOL, 0, sizeof(uint32_t), st);
@@ -398,21 +471,19 @@ int tds_launch_colouring(const DevPtrs &d, uint32_t n, uint32_t cap, int coop_bl
   cudaLaunchCooperativeKernel((const void *)k_colour_rounds, dim3(coop_blocks), dim3(coop_threads),
                               args, 0, st);
   k_colour_masks<<<(n + 255) / 256 < 152 * 16 ? (n + 255) / 256 : 152 * 16, 256, 0, st>>>(d, n);
-  return 5 + scans;
+  return 4 + scans;
 }
 
 // Contact rows (and initial impulses) into the padded colour order.
 int tds_launch_bucketing(const DevPtrs &d, uint32_t cap, cudaStream_t st) {
   int scans = 0;
-  k_bucket_hist<<<d.ntiles, 256, 0, st>>>(d);
-  scans += tds_scan_exclusive(d.tile_hist, d.tile_off, TDS_NBUCKETS * d.ntiles, d.scan_tmp, st);
-  k_bucket_starts<<<1, 32, 0, st>>>(d);
-  cudaMemsetAsync(d.order, 0xFF, sizeof(uint32_t) * ((size_t)cap + TDS_ORDER_PAD), st);
-  cudaMemsetAsync(d.p_ab, 0xFF, sizeof(uint2) * ((size_t)cap + TDS_ORDER_PAD), st);  // padding sentinel
+  k_bucket_hist<<<d.ntiles, kBucketThreads, 0, st>>>(d);
+  scans += tds_scan_exclusive(d.tile_hist, d.tile_off, TDS_NBUCKETS * d.ntiles, d.scan_tmp, st, d.ctr + CTR_HIST);
+  k_bucket_starts<<<1, TDS_NBUCKETS, 0, st>>>(d);
   if (d.nscenes > 1) cudaMemsetAsync(d.scq_cnt, 0, sizeof(uint32_t) * (size_t)d.nscenes * TDS_NBUCKETS, st);
-  k_bucket_scatter<<<d.ntiles, 256, 0, st>>>(d);
-  k_scene_chunks<<<1, 1024, 0, st>>>(d);
-  return 4 + scans;
+  k_bucket_scatter<<<d.ntiles, kBucketThreads, 0, st>>>(d);
+  if (d.nscenes > 1) k_scene_chunks<<<1, 1024, 0, st>>>(d);
+  return 3 + (d.nscenes > 1) + scans;
 }
 
 const void *tds_colour_kernel() { return (const void *)k_colour_rounds; }

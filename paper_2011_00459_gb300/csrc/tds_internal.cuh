@@ -104,7 +104,7 @@ struct DevPtrs {
   float4 *pos2, *pv2;         // reorder targets
   uint32_t *pid2, *sid2;
   // grid
-  uint32_t *cell_of, *cell_count, *cell_start, *cell_cursor, *perm;
+  uint32_t *cell_of, *cell_count, *cell_start, *perm;
   // contacts in owner order (owner = the particle with the smaller id)
   uint32_t *cnt, *cstart;     // per slot (n + 1)
   uint2 *c_ab;                // slot a, slot b | TDS_STATIC + surface id
@@ -115,13 +115,13 @@ struct DevPtrs {
   float4 *c_la;               // initial impulses (n, t1, t2, r.x)
   float2 *c_lb;               // (r.y, r.z)
   // colouring
-  uint32_t *inc_cnt, *inc_start, *inc_cursor;
+  uint32_t *inc_cnt, *inc_start;
   uint2 *inc_ent;             // (contact id, high word of its priority) per incidence
   unsigned long long *prio;   // colouring priority per contact
   uint8_t *colour;
   ulonglong2 *cmask;          // per slot: the colours of its contacts, a bit each
   int32_t *wait;
-  uint32_t *frontier0, *frontier1;
+  uint32_t *frontier0, *frontier1;  // before the colouring: a contact's place among its two particles' incidences
   // bucketing into colour order
   uint32_t *tile_hist, *tile_off, *order;
   uint32_t *bstart, *bend, *bpad;  // padded colour-order range of each bucket
@@ -183,7 +183,8 @@ struct DevPtrs {
 
 enum { CTR_NC = 0, CTR_NCOL = 1, CTR_ITERS = 2, CTR_FCOUNT = 4, /* 4,5,6 */ CTR_NPP = 8,
        CTR_NSTAT = 9, CTR_TOTAL = 10, CTR_ROUNDS = 11, CTR_PADDED = 12, CTR_IMPACTS = 13,
-       CTR_NEW = 14, CTR_SPAWN = 15, CTR_CLEAN = 16, CTR_NCHUNK = 17, CTR_COUNT = 18 };
+       CTR_NEW = 14, CTR_SPAWN = 15, CTR_CLEAN = 16, CTR_NCHUNK = 17, CTR_HIST = 18, CTR_TICKET = 19,
+       CTR_COUNT = 20 };
 enum { FS_RESID = 0, FS_COUNT = 4 };
 // ACC_SWEEP_PP / ACC_SWEEP_ST: sum over steps of sweeps x particle-pair /
 // static contacts (the solver's algorithmic work); ACC_STEPS: steps summed.
@@ -322,6 +323,6 @@ __device__ __forceinline__ bool grid_barrier(uint32_t *bar, int32_t *err, uint32
 }
 
 // Host-side launchers implemented in the .cu files (the scan returns its launches).
-int tds_scan_exclusive(const uint32_t *in, uint32_t *out, uint32_t m, uint32_t *tmp,
-                        cudaStream_t st);
+int tds_scan_exclusive(const uint32_t *in, uint32_t *out, uint32_t m, uint32_t *tmp, cudaStream_t st,
+                       const uint32_t *m_dev = nullptr);
 size_t tds_scan_tmp_words(uint32_t m);

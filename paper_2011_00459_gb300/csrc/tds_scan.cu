@@ -85,7 +85,10 @@ __device__ __forceinline__ uint32_t sum_items(const uint32_t (&v)[kItems]) {
 }
 
 // (in and out may be the same array: no restrict)
-__global__ void __launch_bounds__(kOneThreads) k_scan_one(const uint32_t *in, uint32_t m, uint32_t *out, bool vec) {
+// (m_dev, if not null: the length, known on the device only; m is then its bound)
+__global__ void __launch_bounds__(kOneThreads) k_scan_one(const uint32_t *in, uint32_t m, const uint32_t *m_dev,
+                                                          uint32_t *out, bool vec) {
+  if (m_dev) m = min(m, *m_dev);
   uint32_t carry = 0;
   for (uint32_t start = 0; start < m; start += kOneThreads * kItems) {
     const size_t base = start + (size_t)threadIdx.x * kItems;
@@ -98,16 +101,20 @@ __global__ void __launch_bounds__(kOneThreads) k_scan_one(const uint32_t *in, ui
   if (threadIdx.x == 0) out[m] = carry;
 }
 
-__global__ void __launch_bounds__(kThreads) k_tile_sums(const uint32_t *__restrict__ in, uint32_t m, bool vec,
-                                                        uint32_t *__restrict__ sums) {
+__global__ void __launch_bounds__(kThreads) k_tile_sums(const uint32_t *__restrict__ in, uint32_t m,
+                                                        const uint32_t *m_dev, bool vec, uint32_t *__restrict__ sums) {
+  if (m_dev) m = min(m, *m_dev);
+  if (blockIdx.x > 0 && (size_t)blockIdx.x * kTile >= m) return;
   uint32_t v[kItems], total;
   load_items(in, (size_t)blockIdx.x * kTile + threadIdx.x * kItems, m, vec, v);
   (void)block_exclusive<kThreads>(sum_items(v), &total);
   if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(kThreads) k_tile_scan(const uint32_t *in, uint32_t m, bool vec, const uint32_t *sums,
-                                                        uint32_t *out) {
+__global__ void __launch_bounds__(kThreads) k_tile_scan(const uint32_t *in, uint32_t m, const uint32_t *m_dev, bool vec,
+                                                        const uint32_t *sums, uint32_t *out) {
+  if (m_dev) m = min(m, *m_dev);
+  if (blockIdx.x > 0 && (size_t)blockIdx.x * kTile >= m) return;
   const size_t base = (size_t)blockIdx.x * kTile + threadIdx.x * kItems;
   uint32_t v[kItems], before, total, mine = 0;
   load_items(in, base, m, vec, v);
@@ -115,7 +122,7 @@ __global__ void __launch_bounds__(kThreads) k_tile_scan(const uint32_t *in, uint
   (void)block_exclusive<kThreads>(mine, &before);
   const uint32_t run = block_exclusive<kThreads>(sum_items(v), &total) + before;
   store_items(out, base, m, vec, v, run);
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[m] = before + total;
+  if ((size_t)(blockIdx.x + 1) * kTile >= m && threadIdx.x == 0) out[m] = before + total;  // the last tile
 }
 
 }  // namespace
@@ -125,15 +132,16 @@ size_t tds_scan_tmp_words(uint32_t m) { return (size_t)(m + kTile - 1) / kTile +
 // out[0..m] = exclusive prefix sums of in[0..m), out[m] = total. In-place
 // (in == out) is allowed. tmp holds tds_scan_tmp_words(m) words.
 // Returns the kernels launched.
-int tds_scan_exclusive(const uint32_t *in, uint32_t *out, uint32_t m, uint32_t *tmp,
-                        cudaStream_t st) {
+// With m_dev, the length is *m_dev (at most m) and known on the device only.
+int tds_scan_exclusive(const uint32_t *in, uint32_t *out, uint32_t m, uint32_t *tmp, cudaStream_t st,
+                       const uint32_t *m_dev) {
   const bool vec = (((uintptr_t)in | (uintptr_t)out) & 15u) == 0u;
   if (m <= kOneBlock) {
-    k_scan_one<<<1, kOneThreads, 0, st>>>(in, m, out, vec);
+    k_scan_one<<<1, kOneThreads, 0, st>>>(in, m, m_dev, out, vec);
     return 1;
   }
   const uint32_t ntiles = (m + kTile - 1) / kTile;
-  k_tile_sums<<<ntiles, kThreads, 0, st>>>(in, m, vec, tmp);
-  k_tile_scan<<<ntiles, kThreads, 0, st>>>(in, m, vec, tmp, out);
+  k_tile_sums<<<ntiles, kThreads, 0, st>>>(in, m, m_dev, vec, tmp);
+  k_tile_scan<<<ntiles, kThreads, 0, st>>>(in, m, m_dev, vec, tmp, out);
   return 2;
 }

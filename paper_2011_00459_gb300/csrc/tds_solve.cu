@@ -207,19 +207,6 @@ __device__ __forceinline__ void load_pair(const DevPtrs &d, const Row &r, Side &
   else B = Side{r.sv, r.sw, 0.f, 0.f};
 }
 
-__device__ __forceinline__ double block_sum(double v, double *sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  if (lane == 0) sh[warp] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-  __syncthreads();
-  return t;  // valid in thread 0
-}
-
 struct SolveArgs {
   uint32_t max_iters, every;
   float tol, sig_t, sig_r;
@@ -765,7 +752,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
     unsigned long long pp = 0ull, sc = 0ull;
     for (uint32_t q = threadIdx.x; q < S; q += blockDim.x) {
       const unsigned long long iq = d.scene_iters[q];
-      for (uint32_t b = 0; b < TDS_NBUCKETS; ++b) {
+      for (uint32_t b = 0; b < 2u * ncol; ++b) {
         const unsigned long long c = d.scq_cnt[(size_t)q * TDS_NBUCKETS + b];
         if (b & 1u) sc += iq * c;
         else pp += iq * c;
@@ -860,8 +847,7 @@ __global__ void __launch_bounds__(512) k_impact(DevPtrs d, ImpactArgs a) {
 }
 
 // Colour order -> owner order warm-start memory: (key's other side,
-// impulses with the tangent in world coordinates); per particle id the range
-// of its owned contacts.
+// impulses with the tangent in world coordinates).
 __global__ void k_writeback(DevPtrs d) {
   if (step_failed(d)) return;
   const uint32_t np = d.ctr[CTR_PADDED];
@@ -886,21 +872,13 @@ __global__ void k_writeback(DevPtrs d) {
   }
 }
 
-__global__ void k_prev_ranges(DevPtrs d, uint32_t n, uint32_t cap) {
-  if (step_failed(d)) return;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    uint32_t s = d.cstart[i], e = d.cstart[i + 1];
-    if (s > cap) s = cap;
-    if (e > cap) e = cap;
-    uint32_t me = d.pid[i];
-    d.prev_first[1][me] = s;
-    d.prev_cnt[1][me] = e - s;
-  }
-}
-
-__global__ void k_integrate(DevPtrs d, StepConsts k) {
+__global__ void k_integrate(DevPtrs d, StepConsts k, uint32_t cap) {
   if (step_failed(d)) return;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < k.n; i += gridDim.x * blockDim.x) {
+    // the range of the particle's own contacts in the warm-start memory
+    const uint32_t me = d.pid[i], s = min(d.cstart[i], cap), e = min(d.cstart[i + 1], cap);
+    d.prev_first[1][me] = s;
+    d.prev_cnt[1][me] = e - s;
     // the solved velocities come back from the solver's records
     const float im = d.pv[2 * i].w, iI = d.pv[2 * i + 1].w;
     float4 p = d.pos[i], v = d.rec[2 * (size_t)i], w = d.rec[2 * (size_t)i + 1];
@@ -918,18 +896,52 @@ __global__ void k_integrate(DevPtrs d, StepConsts k) {
 
 // Soil-on-tool force and torque about the tool origin: sum over tool
 // contacts of (Lambda_n n + Lambda_t) / dt at the contact point, plus the
-// rolling impulse / dt. Fixed block partition + fixed-order sums: the
-// result is reproducible.
-constexpr int kToolBlocks = 128;
-__global__ void k_tool_partial(DevPtrs d, StepConsts k) {
+// rolling impulse / dt. Only the static buckets hold tool contacts (all
+// contacts: 98 us on the 1M bed). Fixed block partition + fixed-order
+// sums, the blocks' added by the last one to finish: the result is
+// reproducible.
+constexpr int kToolBlocks = 64;
+
+// Sums of six values per thread over a block of 256 threads, in threads 0 to 5.
+__device__ __forceinline__ double block_sum6(const double (&v)[6], double (*sh)[6]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    double t = v[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) sh[warp][q] = t;
+  }
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < 6)
+    for (int w = 0; w < 8; ++w) t += sh[w][threadIdx.x];
+  __syncthreads();
+  return t;
+}
+
+__global__ void __launch_bounds__(256) k_tool(DevPtrs d, StepConsts k) {
   if (step_failed(d)) return;
-  __shared__ double sh[8];
-  const uint32_t np = d.ctr[CTR_PADDED];
+  __shared__ double sh[8][6];
+  __shared__ bool last;
+  __shared__ uint32_t first[TDS_MAX_COLOURS + 1], start[TDS_MAX_COLOURS];  // static contacts before a colour's, its range
+  const uint32_t ncol = min(d.ctr[CTR_NCOL], (uint32_t)TDS_MAX_COLOURS);
+  for (uint32_t c = threadIdx.x; c < ncol; c += blockDim.x) {
+    start[c] = d.bstart[2 * c + 1];
+    first[c + 1] = d.bend[2 * c + 1] - start[c];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    first[0] = 0u;
+    for (uint32_t c = 0; c < ncol; ++c) first[c + 1] += first[c];
+  }
+  __syncthreads();
   double acc[6] = {0, 0, 0, 0, 0, 0};
-  for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x) {
-    if (d.order[p] == 0xFFFFFFFFu) continue;  // padding slot
+  uint32_t col = 0;
+  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < first[ncol]; t += gridDim.x * blockDim.x) {
+    while (t >= first[col + 1]) ++col;
+    const uint32_t p = start[col] + (t - first[col]);
     uint2 ab = d.p_ab[p];
-    if (is_dyn(ab.y)) continue;
     const uint32_t sid = d.sid[ab.x];
     const SceneGeo &G = k.geo[sid];
     if ((ab.y & ~TDS_STATIC) < 1u + G.nwall) continue;
@@ -950,24 +962,26 @@ __global__ void k_tool_partial(DevPtrs d, StepConsts k) {
     acc[0] += F.x; acc[1] += F.y; acc[2] += F.z;
     acc[3] += T.x; acc[4] += T.y; acc[5] += T.z;
   }
-  for (int q = 0; q < 6; ++q) {
-    double t = block_sum(acc[q], sh);
-    if (threadIdx.x == 0) d.dpart[6 * blockIdx.x + q] = t;
+  if (k.nscenes == 1) {
+    const double s = block_sum6(acc, sh);
+    if (threadIdx.x < 6) __stcg(d.dpart + 6 * blockIdx.x + threadIdx.x, s);
   }
-}
-
-__global__ void k_tool_final(DevPtrs d, uint32_t nscenes) {
-  if (step_failed(d)) return;
-  if (nscenes == 1) {
-    if (threadIdx.x < 6) {
-      double t = 0.0;
-      for (int b = 0; b < kToolBlocks; ++b) t += d.dpart[6 * b + threadIdx.x];
-      d.tool_out[threadIdx.x] = (float)t;
-    }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(d.ctr + CTR_TICKET, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (threadIdx.x == 0) d.ctr[CTR_TICKET] = 0u;  // for the next step
+  if (k.nscenes == 1) {
+#pragma unroll
+    for (int q = 0; q < 6; ++q) acc[q] = threadIdx.x < kToolBlocks ? __ldcg(d.dpart + 6 * threadIdx.x + q) : 0.0;
+    const double s = block_sum6(acc, sh);
+    if (threadIdx.x < 6) d.tool_out[threadIdx.x] = (float)s;
     return;
   }
-  for (uint32_t q = threadIdx.x; q < 6 * nscenes; q += blockDim.x) {
-    d.tool_out[q] = (float)d.tool_acc[q];
+  for (uint32_t q = threadIdx.x; q < 6 * k.nscenes; q += blockDim.x) {
+    d.tool_out[q] = (float)__ldcg(d.tool_acc + q);
     d.tool_acc[q] = 0.0;
   }
 }
@@ -1063,11 +1077,9 @@ int tds_pgs_occupancy(int i) { return g_pgs_occupancy[i]; }
 
 int tds_launch_finish(const DevPtrs &d, const StepConsts &k, uint32_t cap, cudaStream_t st) {
   k_writeback<<<grid_for(cap, 256), 256, 0, st>>>(d);
-  k_prev_ranges<<<grid_for(k.n, 256), 256, 0, st>>>(d, k.n, cap);
-  k_tool_partial<<<kToolBlocks, 256, 0, st>>>(d, k);
-  k_tool_final<<<1, 256, 0, st>>>(d, k.nscenes);
-  k_integrate<<<grid_for(k.n, 256), 256, 0, st>>>(d, k);
-  return 5;
+  k_tool<<<kToolBlocks, 256, 0, st>>>(d, k);
+  k_integrate<<<grid_for(k.n, 256), 256, 0, st>>>(d, k, cap);
+  return 3;
 }
 
 void tds_launch_stage(const DevPtrs &d, uint32_t n, cudaStream_t st) {
