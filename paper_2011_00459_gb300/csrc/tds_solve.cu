@@ -512,17 +512,19 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       if (ntile > 1) load_sides(ring_p + st * kTileBytes);
       uint32_t want_a = 0, want_b = 0;
       bool need_a = live, need_b = live && dyn;
+      Row r;
+      float4 im;
       Pre pre;
       if (live) {
         const uint32_t rk = reinterpret_cast<const uint32_t *>(stage + kOffRk * 32)[lane];
         want_a = passes * ((rk >> 8) & 0xFFu) + (rk & 0xFFu);
         want_b = passes * (rk >> 24) + ((rk >> 16) & 0xFFu);
         // computed while the records are on their way (the empty asm keeps it here)
-        const float4 rn = *s_rn, rq = *s_rq, im = *s_im;
-        Row r;
-        Side A, B;
+        const float4 rn = *s_rn, rq = *s_rq;
+        im = *s_im;
         r.n = f3(rn); r.la = rn.w;
-        r.lb = rq.x; r.Sn = rq.z;
+        r.lb = rq.x; r.qn = rq.y; r.Sn = rq.z; r.fc = rq.w;
+        Side A, B;
         A.im = im.x; A.iI = im.y; B.im = im.z; B.iI = im.w;
         pre = prepare_update(r, A, B, a.sig_t, a.sig_r);
         asm volatile("" : "+f"(pre.iDn), "+f"(pre.iDt), "+f"(pre.iDr), "+f"(pre.t1.x), "+f"(pre.t1.y), "+f"(pre.t1.z),
@@ -531,46 +533,47 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       // Wait for the versions the tile needs (bounded, as every wait). Every
       // lane that needs one reads again; while some record has two or more
       // updates to come, only the lane with the most of them polls.
-      unsigned long long t0 = 0;
-      uint32_t lead = 33u;  // the polling lane; 32: every lane has just read, 33: nothing read again yet
-      for (unsigned spins = 0;; ++spins) {
-        uint32_t behind = 0;
-        if (need_a) {
-          need_a = !is_version(va, wa, want_a);
-          if (need_a) behind = max(1u, want_a - __float_as_uint(va.w));
-        }
-        if (need_b) {
-          need_b = !is_version(vb, wb, want_b);
-          if (need_b) behind = max(max(behind, 1u), want_b - __float_as_uint(vb.w));
-        }
-        if (dead || !__any_sync(0xffffffffu, behind != 0u)) break;
-        if ((spins & 15u) == 15u) {
-          const unsigned long long t = global_ns();
-          if (t0 == 0) t0 = t;
-          else if (t - t0 > d.wait_ns) latch_error(d.err, DEV_ERR_BARRIER);
-          dead = __any_sync(0xffffffffu, *(volatile int32_t *)d.err != 0);
-        }
-        if (lead == 32u) {
-          const uint32_t worst = __reduce_max_sync(0xffffffffu, (min(behind, 0xFFFFFu) << 5) | lane);
-          if (worst >= 64u) lead = worst & 31u;
-        } else if (lead == 33u || __shfl_sync(0xffffffffu, behind, lead) < 2u) {
-          lead = 32u;
-        }
-        if (lead == 32u || lane == lead) {
-          if (need_a) ld_rec(rec_a, va, wa);
-          if (need_b) ld_rec(rec_b, vb, wb);
+      if (need_a) need_a = !is_version(va, wa, want_a);
+      if (need_b) need_b = !is_version(vb, wb, want_b);
+      if (__any_sync(0xffffffffu, need_a || need_b)) {
+        unsigned long long t0 = 0;
+        uint32_t lead = 32u;  // the polling lane; 32: every lane reads
+        for (unsigned spins = 0;; ++spins) {
+          if (lead == 32u || lane == lead) {
+            if (need_a) ld_rec(rec_a, va, wa);
+            if (need_b) ld_rec(rec_b, vb, wb);
+          }
+          uint32_t behind = 0;
+          if (need_a) {
+            need_a = !is_version(va, wa, want_a);
+            if (need_a) behind = max(1u, want_a - __float_as_uint(va.w));
+          }
+          if (need_b) {
+            need_b = !is_version(vb, wb, want_b);
+            if (need_b) behind = max(max(behind, 1u), want_b - __float_as_uint(vb.w));
+          }
+          if (!__any_sync(0xffffffffu, behind != 0u)) break;
+          if (lead == 32u) {
+            const uint32_t worst = __reduce_max_sync(0xffffffffu, (min(behind, 0xFFFFFu) << 5) | lane);
+            if (worst >= 64u) lead = worst & 31u;
+          } else if (__shfl_sync(0xffffffffu, behind, lead) < 2u) {
+            lead = 32u;
+          }
+          if ((spins & 15u) == 15u) {
+            const unsigned long long t = global_ns();
+            if (t0 == 0) t0 = t;
+            else if (t - t0 > d.wait_ns) latch_error(d.err, DEV_ERR_BARRIER);
+            dead = __any_sync(0xffffffffu, *(volatile int32_t *)d.err != 0);
+            if (dead) break;
+          }
         }
       }
       if (live && !dead) {
-        const float4 rn = *s_rn, rq = *s_rq, im = *s_im;
         const float2 rm = reinterpret_cast<const float2 *>(stage + kOffRm * 32)[lane];
         float4 &s_la = reinterpret_cast<float4 *>(stage + kOffLa * 32)[lane];
         float2 &s_lb = reinterpret_cast<float2 *>(stage + kOffLb * 32)[lane];
         float4 L0 = s_la;
         float2 L1 = s_lb;
-        Row r;
-        r.n = f3(rn); r.la = rn.w;
-        r.lb = rq.x; r.qn = rq.y; r.Sn = rq.z; r.fc = rq.w;
         r.mu = rm.x; r.rmu = rm.y;
         Side A{f3(va), f3(wa), im.x, im.y}, B{f3(vb), f3(wb), im.z, im.w};
         if (warm_pass) {  // v = M^-1 (p + G^T lambda_0)
