@@ -62,19 +62,18 @@ __device__ __forceinline__ Row load_row(const DevPtrs &d, uint32_t p) {
 // Projections on the Coulomb disk / rolling ball of radius bound (a zero
 // bound forces zero). All solver arithmetic below spells out its rounding
 // (see the vector helpers): every launch shape of the solver computes the
-// same bits.
+// same bits. Without a branch: inside the bound the factor is 1, which leaves
+// every value as it is.
+__device__ __forceinline__ float shrink(float m2, float bound) {
+  const float s = bound > 0.f ? __fmul_rn(bound, rsqrtf(m2)) : 0.f;
+  return m2 > __fmul_rn(bound, bound) ? s : 1.f;
+}
 __device__ __forceinline__ void disk(float &a, float &b, float bound) {
-  const float m2 = __fmaf_rn(b, b, __fmul_rn(a, a));
-  if (m2 > __fmul_rn(bound, bound)) {
-    const float s = bound > 0.f ? __fmul_rn(bound, rsqrtf(m2)) : 0.f;
-    a = __fmul_rn(a, s);
-    b = __fmul_rn(b, s);
-  }
+  const float s = shrink(__fmaf_rn(b, b, __fmul_rn(a, a)), bound);
+  a = __fmul_rn(a, s);
+  b = __fmul_rn(b, s);
 }
-__device__ __forceinline__ void ball(float3 &a, float bound) {
-  const float m2 = dot(a, a);
-  if (m2 > __fmul_rn(bound, bound)) a = (bound > 0.f ? __fmul_rn(bound, rsqrtf(m2)) : 0.f) * a;
-}
+__device__ __forceinline__ void ball(float3 &a, float bound) { a = shrink(dot(a, a), bound) * a; }
 
 // v += M^-1 G^T dLambda for each row group. A static side has zero inverse
 // mass and inertia, so its (discarded) update is a no-op.
@@ -513,7 +512,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       uint32_t want_a = 0, want_b = 0;
       bool need_a = live, need_b = live && dyn;
       Row r;
-      float4 im;
+      float4 im, L0;
+      float2 L1;
       Pre pre;
       if (live) {
         const uint32_t rk = reinterpret_cast<const uint32_t *>(stage + kOffRk * 32)[lane];
@@ -524,6 +524,10 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
         im = *s_im;
         r.n = f3(rn); r.la = rn.w;
         r.lb = rq.x; r.qn = rq.y; r.Sn = rq.z; r.fc = rq.w;
+        const float2 rm = reinterpret_cast<const float2 *>(stage + kOffRm * 32)[lane];
+        r.mu = rm.x; r.rmu = rm.y;
+        L0 = reinterpret_cast<const float4 *>(stage + kOffLa * 32)[lane];
+        L1 = reinterpret_cast<const float2 *>(stage + kOffLb * 32)[lane];
         Side A, B;
         A.im = im.x; A.iI = im.y; B.im = im.z; B.iI = im.w;
         pre = prepare_update(r, A, B, a.sig_t, a.sig_r);
@@ -569,12 +573,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
         }
       }
       if (live && !dead) {
-        const float2 rm = reinterpret_cast<const float2 *>(stage + kOffRm * 32)[lane];
         float4 &s_la = reinterpret_cast<float4 *>(stage + kOffLa * 32)[lane];
         float2 &s_lb = reinterpret_cast<float2 *>(stage + kOffLb * 32)[lane];
-        float4 L0 = s_la;
-        float2 L1 = s_lb;
-        r.mu = rm.x; r.rmu = rm.y;
         Side A{f3(va), f3(wa), im.x, im.y}, B{f3(vb), f3(wb), im.z, im.w};
         if (warm_pass) {  // v = M^-1 (p + G^T lambda_0)
           if (!(L0.x == 0.f && L0.y == 0.f && L0.z == 0.f && L0.w == 0.f && L1.x == 0.f && L1.y == 0.f))
