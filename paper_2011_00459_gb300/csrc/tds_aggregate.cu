@@ -4,10 +4,11 @@
 // angular velocity I^+ L of the particles it contains. Two passes, as in the
 // definition: (1) membership, M, sum m x, sum m v; (2) the second moments and
 // angular momentum about the centre of mass. FP64 accumulation in
-// registers (see LaneSums). What bounds the passes: FP64 issue and its
-// latency (20 and 31 operations a particle). 1M particles, 8 zones: 53 and 68
-// us; with five shuffle steps and additions per component and 32 particles,
-// and FP64 divisions, 146 and 185. k_agg_final 6.8 us against 24.
+// registers (see LaneSums). What bounds the passes: FP64 issue (13 and 19
+// operations a particle; an FP64 instruction takes 16 cycles of an SM). 1M
+// particles, 8 zones: 39 and 44 us; with FP64 divisions, conversions and five
+// shuffle steps and additions per component and 32 particles 146 and 185.
+// k_agg_final 6.4 us against 24.
 #include <cstring>
 
 #include "tds_internal.cuh"
@@ -39,13 +40,26 @@ __device__ __forceinline__ int zone_of(const tds_zone *zones, uint32_t nz, uint3
   return -1;
 }
 
+// An FP32 number as FP64, exactly, by integer operations: the conversion
+// instruction takes an FP64 issue slot, worth 64 integer ones here. Zeros and
+// denormals are scaled up first; infinities and NaN keep their exponent.
+__device__ __forceinline__ double widen(float x) {
+  const bool tiny = (__float_as_uint(x) & 0x7F800000u) == 0u;
+  const uint32_t u = __float_as_uint(tiny ? __fmul_rn(x, 18446744073709551616.0f) : x);  // 2^64
+  const uint32_t mag = u & 0x7FFFFFFFu;
+  uint32_t hi = (mag >> 3) + (tiny ? (896u - 64u) << 20 : 896u << 20);
+  if (mag == 0u) hi = 0u;
+  if (mag >= 0x7F800000u) hi = 0x7FF00000u | ((mag & 0x7FFFFFu) >> 3);
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
+
 // Mass of a particle: the reciprocal of the FP32 record's 1/m. FP64 division
 // costs about twenty FP64 operations, which this GPU issues at a sixty-fourth
 // of the FP32 rate; Newton's iteration r <- r + r (1 - a r) doubles the correct
 // digits of the FP32 reciprocal, to 2^-46 and then to the last bit.
 __device__ __forceinline__ double mass_of(float inv_m) {
-  const double a = (double)inv_m;
-  double r = (double)__frcp_rn(inv_m);
+  const double a = widen(inv_m);
+  double r = widen(__frcp_rn(inv_m));
   r = fma(r, fma(-a, r, 1.0), r);
   return fma(r, fma(-a, r, 1.0), r);
 }
@@ -127,7 +141,7 @@ __device__ __forceinline__ void warp_stretch(uint32_t n, uint32_t &lo, uint32_t 
 
 __global__ void __launch_bounds__(kAggThreads) k_agg_first(DevPtrs d, uint32_t n,
                                                            const __grid_constant__ ZoneTable zones, uint32_t nz,
-                                                           uint8_t *zone_id, double *sums) {
+                                                           uint8_t *zone_id, double *mass, double *sums) {
   __shared__ tds_zone sz[TDS_MAX_ZONES];
   __shared__ double sh[TDS_MAX_ZONES * kFirst];
   for (uint32_t q = threadIdx.x; q < nz * sizeof(tds_zone) / 4; q += blockDim.x)
@@ -148,13 +162,14 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_first(DevPtrs d, uint32_t n
     const float4 v = d.pv[2 * (size_t)i];
     ls.enter(sh, z);
     const double m = mass_of(v.w);
+    mass[i] = m;
     ls.acc[0] += m;
-    ls.acc[1] = fma(m, (double)p.x, ls.acc[1]);
-    ls.acc[2] = fma(m, (double)p.y, ls.acc[2]);
-    ls.acc[3] = fma(m, (double)p.z, ls.acc[3]);
-    ls.acc[4] = fma(m, (double)v.x, ls.acc[4]);
-    ls.acc[5] = fma(m, (double)v.y, ls.acc[5]);
-    ls.acc[6] = fma(m, (double)v.z, ls.acc[6]);
+    ls.acc[1] = fma(m, widen(p.x), ls.acc[1]);
+    ls.acc[2] = fma(m, widen(p.y), ls.acc[2]);
+    ls.acc[3] = fma(m, widen(p.z), ls.acc[3]);
+    ls.acc[4] = fma(m, widen(v.x), ls.acc[4]);
+    ls.acc[5] = fma(m, widen(v.y), ls.acc[5]);
+    ls.acc[6] = fma(m, widen(v.z), ls.acc[6]);
     ls.acc[7] += 1.0;
   }
   ls.finish(sh);
@@ -162,7 +177,7 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_first(DevPtrs d, uint32_t n
 }
 
 __global__ void __launch_bounds__(kAggThreads) k_agg_second(DevPtrs d, uint32_t n, uint32_t nz,
-                                                            const uint8_t *zone_id, const double *first,
+                                                            const uint8_t *zone_id, const double *mass, const double *first,
                                                             double *sums) {
   __shared__ double com[TDS_MAX_ZONES][3];
   __shared__ double sh[TDS_MAX_ZONES * kSecond];
@@ -183,9 +198,9 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_second(DevPtrs d, uint32_t 
     const float4 p = d.pos[i];
     const float4 v = d.pv[2 * (size_t)i];
     ls.enter(sh, z);
-    const double m = mass_of(v.w);
-    const double dx = (double)p.x - com[z][0], dy = (double)p.y - com[z][1], dz = (double)p.z - com[z][2];
-    const double vx = (double)v.x, vy = (double)v.y, vz = (double)v.z;
+    const double m = mass[i];
+    const double dx = widen(p.x) - com[z][0], dy = widen(p.y) - com[z][1], dz = widen(p.z) - com[z][2];
+    const double vx = widen(v.x), vy = widen(v.y), vz = widen(v.z);
     const double mx = m * dx, my = m * dy, mz = m * dz;
     ls.acc[0] = fma(mx, dx, ls.acc[0]);
     ls.acc[1] = fma(my, dy, ls.acc[1]);
@@ -296,17 +311,18 @@ int tds_launch_aggregate(const DevPtrs &d, uint32_t n, const tds_zone *zones, ui
   cudaMemsetAsync(sums, 0, sizeof(double) * TDS_MAX_ZONES * (kFirst + kSecond), st);
   int sms = 152, dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // three blocks per SM (1, 2, 3, 4, 6: 156, 122, 121, 129, 137 us for both
-  // passes over 1M particles; the longer a warp's stretch, the fewer reductions
+  // three blocks per SM (2, 3, 4: 89, 83, 87 us for both passes over
+  // 1M particles; the longer a warp's stretch, the fewer reductions
   // at its end), fewer for small n so that every
   // warp has at least 128 slots
   uint32_t blocks = (n + 128u * (kAggThreads / 32) - 1) / (128u * (kAggThreads / 32));
   if (blocks < 1) blocks = 1;
   if (blocks > (uint32_t)(3 * sms)) blocks = 3 * sms;
+  double *mass = reinterpret_cast<double *>(d.stage);  // of the particles in a zone (read-back scratch)
   ZoneTable table;
   std::memcpy(table.z, zones, sizeof(tds_zone) * nz);
-  k_agg_first<<<blocks, kAggThreads, 0, st>>>(d, n, table, nz, zone_id, first);
-  k_agg_second<<<blocks, kAggThreads, 0, st>>>(d, n, nz, zone_id, first, second);
+  k_agg_first<<<blocks, kAggThreads, 0, st>>>(d, n, table, nz, zone_id, mass, first);
+  k_agg_second<<<blocks, kAggThreads, 0, st>>>(d, n, nz, zone_id, mass, first, second);
   k_agg_final<<<1, TDS_MAX_ZONES, 0, st>>>(nz, first, second, out);
   return 3;
 }
