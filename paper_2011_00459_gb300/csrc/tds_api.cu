@@ -406,11 +406,7 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
   d.bpad = c.take<uint32_t>(TDS_NBUCKETS);
   const size_t pc = (size_t)cap + TDS_ORDER_PAD;  // colour order with padding
   d.order = c.take<uint32_t>(pc);
-  d.p_ab = c.take<uint2>(pc);
-  d.p_rn = c.take<float4>(pc); d.p_rq = c.take<float4>(pc);
-  d.p_rm = c.take<float2>(pc);
-  d.p_im = c.take<float4>(pc);
-  d.p_rk = c.take<uint32_t>(pc);
+  d.p_rows = c.take<unsigned char>((pc / 32 + 1) * sizeof(RowTile));
   d.p_sv = c.take<float4>(pc); d.p_sw = c.take<float4>(pc);
   d.p_la = c.take<float4>(pc); d.p_lb = c.take<float2>(pc);
   d.p_il = c.take<float4>(pc); d.p_il2 = c.take<float4>(pc);

@@ -305,20 +305,23 @@ __device__ __forceinline__ void write_chunks(const DevPtrs &d, uint32_t first, u
 }
 
 // Bucket ranges in the padded colour order: every bucket starts at a multiple
-// of 4 contacts (16-byte aligned rows); padding slots carry
-// order == 0xFFFFFFFF and are never solved. For a single scene also its
+// of 32 contacts (a row tile); padding slots carry order == 0xFFFFFFFF and a
+// row whose ab is all ones, and are never solved. For a single scene also its
 // residual chunks. One block, a thread per bucket (one thread for all of them:
 // 110 us against 4).
 __global__ void __launch_bounds__(TDS_NBUCKETS) k_bucket_starts(DevPtrs d) {
   const uint32_t nc = d.ctr[CTR_NC], nt = used_tiles(nc), nb = used_buckets(d), b = threadIdx.x;
   const uint32_t u0 = b < nb && nt ? d.tile_off[b * nt] : nc, u1 = b + 1u < nb && nt ? d.tile_off[(b + 1u) * nt] : nc;
-  const uint32_t cnt = u1 - u0, padded = (cnt + 3u) & ~3u;
+  const uint32_t cnt = u1 - u0, padded = (cnt + 31u) & ~31u;
   uint32_t total;
   const uint32_t start = block_prefix<TDS_NBUCKETS>(padded, &total);
   d.bstart[b] = start;
   d.bend[b] = start + cnt;
   d.bpad[b] = start - u0;
-  for (uint32_t p = start + cnt; p < start + padded; ++p) d.order[p] = 0xFFFFFFFFu;
+  for (uint32_t p = start + cnt; p < start + padded; ++p) {
+    d.order[p] = 0xFFFFFFFFu;
+    row_tile(d, p).ab[p & 31u] = make_uint2(~0u, ~0u);
+  }
   if (b == 0u) {
     d.bstart[TDS_NBUCKETS] = total;
     d.ctr[CTR_PADDED] = total;
@@ -382,7 +385,6 @@ __global__ void __launch_bounds__(kBucketThreads) k_bucket_scatter(DevPtrs d) {
       const uint32_t p = wcnt[warp][bk] + rank_in_warp;
       const uint2 ab = d.c_ab[c];
       d.order[p] = c;
-      d.p_ab[p] = ab;
       uint32_t rk = rank_degree(d.cmask[ab.x], bk >> 1);
       float4 im = make_float4(d.pv[2 * (size_t)ab.x].w, d.pv[2 * (size_t)ab.x + 1].w, 0.f, 0.f);
       if (is_dyn(ab.y)) {
@@ -390,11 +392,14 @@ __global__ void __launch_bounds__(kBucketThreads) k_bucket_scatter(DevPtrs d) {
         im.z = d.pv[2 * (size_t)ab.y].w;
         im.w = d.pv[2 * (size_t)ab.y + 1].w;
       }
-      d.p_im[p] = im;
-      d.p_rk[p] = rk;
-      d.p_rn[p] = d.c_rn[c];
-      d.p_rq[p] = d.c_rq[c];
-      d.p_rm[p] = d.c_rm[c];
+      RowTile &row = row_tile(d, p);
+      const uint32_t at = p & 31u;
+      row.rn[at] = d.c_rn[c];
+      row.rq[at] = d.c_rq[c];
+      row.im[at] = im;
+      row.ab[at] = ab;
+      row.rm[at] = d.c_rm[c];
+      row.rk[at] = rk;
       if (bk & 1u) { d.p_sv[p] = d.c_sv[c]; d.p_sw[p] = d.c_sw[c]; }
       d.p_la[p] = d.c_la[c];
       d.p_lb[p] = d.c_lb[c];

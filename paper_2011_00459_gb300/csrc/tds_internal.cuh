@@ -11,7 +11,7 @@
 #define TDS_MAX_COLOURS 128
 #define TDS_NBUCKETS (2 * TDS_MAX_COLOURS)  // (colour, static?) buckets
 #define TDS_TILE 2048                       // contacts per bucketing tile
-#define TDS_ORDER_PAD (4 * TDS_NBUCKETS + 16) // padding slots of the colour order
+#define TDS_ORDER_PAD (32 * TDS_NBUCKETS)     // padding slots of the colour order
 #define TDS_RES_CHUNK 256u                  // contacts per residual chunk (at most)
 #define TDS_BARRIER_NS 2000000000ull        // default limit of a wait on other CTAs (2 s); also the
                                             // fixed limit of a CTA's wait for its own bulk copies
@@ -127,11 +127,7 @@ struct DevPtrs {
   uint32_t *bstart, *bend, *bpad;  // padded colour-order range of each bucket
   uint32_t ntiles;
   // colour order (what the solver streams)
-  uint2 *p_ab;
-  float4 *p_rn, *p_rq;
-  float2 *p_rm;
-  float4 *p_im;               // 1/m_a, 1/I_a, 1/m_b, 1/I_b (0 for a static side)
-  uint32_t *p_rk;             // rank and degree of the contact at a, then at b (a byte each)
+  unsigned char *p_rows;      // row tiles of 32 contacts, see RowTile
   float4 *p_sv, *p_sw;
   float4 *p_la;
   float2 *p_lb;
@@ -180,6 +176,21 @@ struct DevPtrs {
 };
 
 
+
+// The rows of 32 consecutive contacts of the colour order, field by field: one
+// bulk copy brings a tile into shared memory. Every bucket starts with a tile;
+// slots past a bucket's end have ab all ones.
+struct alignas(128) RowTile {
+  float4 rn[32];    // (n, la)
+  float4 rq[32];    // (lb, q_n, Sigma_n, f_c)
+  float4 im[32];    // 1/m_a, 1/I_a, 1/m_b, 1/I_b (0 for a static side)
+  uint2 ab[32];     // slot a, slot b | TDS_STATIC + surface id
+  float2 rm[32];    // (mu, rbar mu_r)
+  uint32_t rk[32];  // rank and degree of the contact at a, then at b (a byte each)
+};
+__device__ __forceinline__ RowTile &row_tile(const DevPtrs &d, uint32_t p) {
+  return reinterpret_cast<RowTile *>(d.p_rows)[p >> 5];
+}
 
 enum { CTR_NC = 0, CTR_NCOL = 1, CTR_ITERS = 2, CTR_FCOUNT = 4, /* 4,5,6 */ CTR_NPP = 8,
        CTR_NSTAT = 9, CTR_TOTAL = 10, CTR_ROUNDS = 11, CTR_PADDED = 12, CTR_IMPACTS = 13,

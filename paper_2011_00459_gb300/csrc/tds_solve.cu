@@ -15,6 +15,8 @@
 // rbar mu_r |Lambda_n| (Eqs. signCoul1-3), each followed by
 // v += M^-1 G^T dLambda. Particle velocities are read and written through L2
 // because other SMs update them between colours.
+#include <cstddef>
+
 #include "tds_internal.cuh"
 
 namespace {
@@ -47,9 +49,11 @@ struct Row {
 
 __device__ __forceinline__ Row load_row(const DevPtrs &d, uint32_t p) {
   Row r;
-  r.ab = d.p_ab[p];
-  float4 rn = d.p_rn[p], rq = d.p_rq[p];
-  float2 rm = d.p_rm[p];
+  const RowTile &t = row_tile(d, p);
+  const uint32_t at = p & 31u;
+  r.ab = t.ab[at];
+  float4 rn = t.rn[at], rq = t.rq[at];
+  float2 rm = t.rm[at];
   r.n = f3(rn);
   r.la = rn.w;
   r.lb = rq.x; r.qn = rq.y; r.Sn = rq.z; r.fc = rq.w;
@@ -289,21 +293,57 @@ constexpr uint32_t kFirstCheck = 5;                  // first residual check in 
 constexpr uint32_t kResSum = 256;                    // residual: threads adding up a large scene's chunks
 constexpr uint32_t kWarpChunks = 1024;               // residual: scenes with at most this many chunks
                                                      // are added by one warp, larger ones by the CTA
-// A row tile: the rows and impulses of 32 contacts of one bucket (one lane
-// each), field by field. Per contact: (n, la) 16 | (lb, q_n, Sigma_n, f_c) 16 |
-// (1/m_a, 1/I_a, 1/m_b, 1/I_b) 16 | impulses (n, t1, t2, r.x) 16 | ab 8 |
-// (mu, rbar mu_r) 8 | impulses (r.y, r.z) 8 | ranks and degrees 4 | index 4
-constexpr size_t kRowBytes = 96;
-constexpr size_t kOffRn = 0, kOffRq = 16, kOffIm = 32, kOffLa = 48, kOffAb = 64, kOffRm = 72, kOffLb = 80, kOffRk = 88,
-                 kOffIx = 92;  // x 32 contacts
+// A warp's ring holds row tiles (see RowTile) with their impulses. Per contact:
+// (n, la) 16 | (lb, q_n, Sigma_n, f_c) 16 | (1/m_a, 1/I_a, 1/m_b, 1/I_b) 16 |
+// ab 8 | (mu, rbar mu_r) 8 | ranks and degrees 4 | impulses (n, t1, t2, r.x) 16 |
+// (r.y, r.z) 8
+constexpr size_t kRowBytes = 92;
+constexpr size_t kOffRn = 0, kOffRq = 16, kOffIm = 32, kOffAb = 48, kOffRm = 56, kOffRk = 64, kOffLa = 68,
+                 kOffLb = 84;  // x 32 contacts
+static_assert(sizeof(RowTile) == 32 * kOffLa && offsetof(RowTile, ab) == 32 * kOffAb && offsetof(RowTile, rk) == 32 * kOffRk,
+              "the ring's tiles are row tiles followed by impulses");
 constexpr size_t kTileBytes = 32 * kRowBytes;
 __host__ __device__ constexpr int ring_tiles(int per_thread) { return kStages * per_thread + 1; }
 __host__ __device__ constexpr size_t pgs_smem(int threads, int per_thread) {
-  return (size_t)(threads / 32) * ring_tiles(per_thread) * kTileBytes;
+  return (size_t)(threads / 32) * ring_tiles(per_thread) * (kTileBytes + 8);  // + a barrier per tile
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void mbar_init(uint32_t bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// Bounded wait for a phase of a tile's barrier (its own warp's copy, which
+// completes in microseconds: the fixed limit): false, with the error latched,
+// when it runs out.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t *err) {
+  if (mbar_test(bar, parity)) return true;
+  const unsigned long long t0 = global_ns();
+  while (!mbar_test(bar, parity))
+    if (global_ns() - t0 > TDS_BARRIER_NS) {
+      latch_error(err, DEV_ERR_BARRIER);
+      return false;
+    }
+  return true;
+}
+// One lane: the row tile into shared memory, counted by the barrier.
+__device__ __forceinline__ void bulk_rows(uint32_t dst, const RowTile *src, uint32_t bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)sizeof(RowTile))
+               : "memory");
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+      "r"((uint32_t)sizeof(RowTile)), "r"(bar)
+      : "memory");
 }
 template <int B>
 __device__ __forceinline__ void cp_async(uint32_t dst, const void *src) {
@@ -314,24 +354,11 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// One lane copies its own contact's row; only that lane reads it, so its own
-// wait for the copy is all the synchronisation there is.
-__device__ __forceinline__ void stage_row(const DevPtrs &d, uint32_t p, uint32_t stage, uint32_t lane) {
-  cp_async<16>(stage + kOffRn * 32 + 16 * lane, d.p_rn + p);
-  cp_async<16>(stage + kOffRq * 32 + 16 * lane, d.p_rq + p);
-  cp_async<16>(stage + kOffIm * 32 + 16 * lane, d.p_im + p);
-  cp_async<16>(stage + kOffLa * 32 + 16 * lane, d.p_la + p);
-  cp_async<8>(stage + kOffAb * 32 + 8 * lane, d.p_ab + p);
-  cp_async<8>(stage + kOffRm * 32 + 8 * lane, d.p_rm + p);
-  cp_async<8>(stage + kOffLb * 32 + 8 * lane, d.p_lb + p);
-  cp_async<4>(stage + kOffRk * 32 + 4 * lane, d.p_rk + p);
-}
-
 // The row and both sides of contact p as the residual pass reads them (after
 // a grid barrier: no update is in flight).
 __device__ __forceinline__ Row settled_pair(const DevPtrs &d, uint32_t p, Side &A, Side &B) {
   Row r = load_row(d, p);
-  const float4 im = d.p_im[p];
+  const float4 im = row_tile(d, p).im[p & 31u];
   float4 v, w;
   ld_rec(d.rec + 2 * (size_t)r.ab.x, v, w);
   A = Side{f3(v), f3(w), im.x, im.y};
@@ -346,29 +373,34 @@ __device__ __forceinline__ Row settled_pair(const DevPtrs &d, uint32_t p, Side &
 
 // The persistent solver. The colour order is cut into row tiles of 32
 // contacts, dealt out to the warps in turn. A warp runs through its tiles
-// sweep after sweep without any barrier: rows and impulses arrive in a ring of
-// shared memory (cp.async, or stay there when the ring holds all of the warp's
-// tiles), the particle records of the next tile are read while this one is
-// solved, and a contact waits only for the versions of its two particles. Grid
-// barriers remain around residual checks.
+// sweep after sweep without any barrier: a tile's rows arrive in a ring of
+// shared memory as one bulk copy, its impulses by a copy of each lane (or both
+// stay there when the ring holds all of the warp's tiles), the particle
+// records of the next tile are read while this one is solved, and a contact
+// waits only for the versions of its two particles. Grid barriers remain
+// around residual checks.
 //
 // What bounds it: on beds of a few thousand tiles the chain of dependent
-// updates (about 2.5 us of L2 round trips and arithmetic from one update of a
-// particle to the next); on the largest beds the L1 data pipe (a record is one
-// wavefront per lane and access) and the rows' DRAM traffic. Measured against
-// the solver this replaced (rows staged by a TMA warp, every colour a
-// barrier between neighbouring CTAs), same box, ms for 100 sweeps: 1M spheres
-// (3.2M contacts) 8.84 against 12.1, 200k 2.88 against 5.76, 50k 1.92 against
-// 3.34; 2000 spheres, 50 sweeps 0.61 against 1.18; 64 beds of 406k spheres in
-// all, 50 sweeps 1.49 against 2.64.
+// updates (1.1 to 1.3 us of L2 round trips and arithmetic from one update of a
+// particle to the next, a read taking about 850 cycles); on the largest beds
+// the L1 data pipe (a record is one wavefront per lane and access), L2 and the
+// rows' DRAM traffic about equally. Measured against the solver this replaced
+// (rows staged by a TMA warp, every colour a barrier between neighbouring
+// CTAs), same box, ms for 100 sweeps: 1M spheres (3.2M contacts) 8.57 against
+// 12.1, 200k 2.55 against 5.76, 50k 1.61 against 3.34; 2000 spheres, 50 sweeps
+// 0.51 against 1.18; 64 beds of 406k spheres in all, 50 sweeps 1.34 against
+// 2.64.
 //  - 16 warps an SM with 128 registers each: 26 warps with 72 registers spill,
-//    and spilling took half of the L1 traffic (1M spheres 17.2 ms).
+//    and spilling took half of the L1 traffic (1M spheres 17.2 ms); 20 or 24
+//    warps that do not read records ahead 8.99 and 9.92 against 8.77.
 //  - Tiles in turn rather than a stretch of slots per warp: every warp gets the
 //    same number (2000 spheres 0.70 against 1.48 ms), and dependent tiles are
 //    a whole colour apart.
 //  - One lane polls while a record is two or more updates away: polling with
 //    every lane of every waiting warp saturates L2 (50k spheres 4.42 against
 //    2.69 ms).
+//  - Rows by one bulk copy a tile rather than six copies of each lane: 8.57
+//    against 8.77 ms at 1M, 1.61 against 1.68 at 50k.
 template <int kThreads, int kPerThread, int kMinBlocks>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveArgs a) {
   constexpr int kRing = ring_tiles(kPerThread);  // tiles in a warp's ring
@@ -418,8 +450,15 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
   const uint32_t ntile = warp < total ? (total - warp + nwarps - 1u) / nwarps : 0u;
   const uint2 *list = d.tiles + warp;
 
+  // (the ring's tiles stay 128-byte aligned: the barriers come after all of them)
   const uint32_t ring = smem_u32(smem) + (threadIdx.x >> 5) * (uint32_t)(kRing * kTileBytes);
   unsigned char *ring_p = smem + (size_t)(threadIdx.x >> 5) * (kRing * kTileBytes);
+  const uint32_t bars = smem_u32(smem) + (kThreads / 32) * (uint32_t)(kRing * kTileBytes) + (threadIdx.x >> 5) * (kRing * 8u);
+  if (lane == 0) {
+    for (int k = 0; k < kRing; ++k) mbar_init(bars + 8u * k);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncwarp();
   // lane l keeps entry l of the list's current group of 32
   uint2 ent = lane < ntile ? list[(size_t)lane * nwarps] : make_uint2(0u, 0u);
   uint32_t group = 0;
@@ -440,28 +479,55 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
   bool dead = false;  // this warp's wait gave up (the error is latched)
   uint32_t it = 0;
   uint32_t fetch = 0, fst = 0, st = 0;  // next tile to fetch, its ring stage, the current tile's stage
+  uint32_t fetched = 0, taken = 0;      // tiles fetched, and waited for, since the start
+  uint32_t tst = 0, tparity = 0;        // the next tile to wait for: its stage, its barrier's phase
+  uint32_t first_of[kAhead + 1];        // first contact of the current tile and the ones fetched after it
   auto fetch_next = [&](bool on) {
     if (on) {
-      const uint2 e = entry(fetch);
-      const uint32_t stage = ring + fst * (uint32_t)kTileBytes;
-      const bool mine = lane < (e.y & 0xFFu);
-      reinterpret_cast<uint32_t *>(ring_p + fst * kTileBytes + kOffIx * 32)[lane] = mine ? e.x + lane : ~0u;
-      if (mine) stage_row(d, e.x + lane, stage, lane);
+      const uint32_t p0 = entry(fetch).x, stage = ring + fst * (uint32_t)kTileBytes;
+      first_of[kAhead] = p0;
+      __syncwarp();  // every lane has read what the stage held
+      if (lane == 0) bulk_rows(stage, &row_tile(d, p0), bars + 8u * fst);
+      cp_async<16>(stage + kOffLa * 32 + 16 * lane, d.p_la + p0 + lane);
+      cp_async<8>(stage + kOffLb * 32 + 8 * lane, d.p_lb + p0 + lane);
       if (++fetch == ntile) fetch = 0;
       if (++fst == stages) fst = 0;
+      ++fetched;
     }
     cp_commit();
   };
-  for (int k = 0; k < kAhead; ++k) fetch_next(ntile > 0 && (!resident || k < (int)ntile));
+  // every tile fetched is waited for in turn (a stage's barrier completes a
+  // phase per tile); resident tiles once
+  auto take_rows = [&](uint32_t upto) {
+    bool ok = true;
+    while (taken < min(upto, fetched) && ok) {
+      ok = __all_sync(0xffffffffu, mbar_wait(bars + 8u * tst, tparity, d.err));
+      ++taken;
+      if (++tst == stages) {
+        tst = 0;
+        tparity ^= 1u;
+      }
+    }
+    return ok;
+  };
+  // before the CTA gives up its shared memory: all copies into it have landed
+  auto drain = [&] {
+    cp_wait<0>();
+    while (taken < fetched) (void)take_rows(fetched);  // (a wait that runs out counts as taken)
+  };
+#pragma unroll
+  for (int k = 0; k < kAhead; ++k) {
+    fetch_next(ntile > 0 && (!resident || k < (int)ntile));
+    first_of[k] = first_of[kAhead];
+  }
   // The records of a tile are read one tile ahead: whether they hold the
   // versions it needs is looked at when its turn comes, and only those that
   // did not are read again.
   float4 nva, nwa, nvb, nwb;
   nva = nwa = nvb = nwb = make_float4(0.f, 0.f, 0.f, 0.f);
-  auto load_sides = [&](const unsigned char *stage) {
-    const uint32_t p = reinterpret_cast<const uint32_t *>(stage + kOffIx * 32)[lane];
-    if (p == ~0u) return;
+  auto load_sides = [&](const unsigned char *stage, uint32_t p) {  // p: the lane's contact
     const uint2 ab = reinterpret_cast<const uint2 *>(stage + kOffAb * 32)[lane];
+    if (ab.x == ~0u) return;
     ld_rec(d.rec + 2 * (size_t)ab.x, nva, nwa);
     if (is_dyn(ab.y)) {
       ld_rec(d.rec + 2 * (size_t)ab.y, nvb, nwb);
@@ -470,8 +536,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       nwb = __ldg(d.p_sw + p);
     }
   };
-  cp_wait<kAhead - 1>();
-  if (ntile > 0) load_sides(ring_p);
+  dead = !take_rows(1);
+  if (ntile > 0 && !dead) load_sides(ring_p, entry(0).x + lane);
 
   // residual checks: every `every` sweeps, or (every == 0) where the decay
   // seen so far says the tolerance will be met (see below)
@@ -488,27 +554,29 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       if (!a.sync)  // grid barrier after every colour
         for (const uint32_t c = entry(j).y >> 9; col < c; ++col)
           if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) {
-            cp_wait<0>();
+            drain();
             return;
           }
       fetch_next(!resident || (passes == 0 && kAhead + j < ntile));
-      cp_wait<kAhead - 1>();  // this tile's rows and the next one's are here
+      cp_wait<kAhead>();  // this tile's impulses are here
+      dead = !take_rows(resident ? ntile : taken + 1u);  // and the next tile's rows
+      if (dead) break;
       unsigned char *stage = ring_p + st * kTileBytes;
       if (++st == stages) st = 0;
-      const uint32_t p = reinterpret_cast<const uint32_t *>(stage + kOffIx * 32)[lane];
+      const uint32_t p = (resident ? entry(j).x : first_of[0]) + lane;
+      const uint32_t p_next = (resident ? entry(j + 1 == ntile ? 0 : j + 1).x : first_of[1]) + lane;
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) first_of[k] = first_of[k + 1];
       const float4 *s_rn = reinterpret_cast<const float4 *>(stage + kOffRn * 32) + lane;
       const float4 *s_rq = reinterpret_cast<const float4 *>(stage + kOffRq * 32) + lane;
       const float4 *s_im = reinterpret_cast<const float4 *>(stage + kOffIm * 32) + lane;
-      uint2 ab = make_uint2(0u, TDS_STATIC);
-      bool live = p != ~0u;
-      if (live) {
-        ab = reinterpret_cast<const uint2 *>(stage + kOffAb * 32)[lane];
-        live = !skip_done || !scene_done(s_done, __ldcg(d.sid + ab.x));
-      }
+      const uint2 ab = reinterpret_cast<const uint2 *>(stage + kOffAb * 32)[lane];
+      bool live = ab.x != ~0u;
+      if (live && skip_done) live = !scene_done(s_done, __ldcg(d.sid + ab.x));
       const bool dyn = is_dyn(ab.y);
       float4 *rec_a = d.rec + 2 * (size_t)ab.x, *rec_b = d.rec + 2 * (size_t)ab.y;
       float4 va = nva, wa = nwa, vb = nvb, wb = nwb;
-      if (ntile > 1) load_sides(ring_p + st * kTileBytes);
+      if (ntile > 1) load_sides(ring_p + st * kTileBytes, p_next);
       uint32_t want_a = 0, want_b = 0;
       bool need_a = live, need_b = live && dyn;
       Row r;
@@ -593,12 +661,12 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
           }
         }
       }
-      if (ntile == 1) load_sides(stage);
+      if (ntile == 1) load_sides(stage, p);
     }
     if (!a.sync)
       for (; col < ncol; ++col)
         if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) {
-          cp_wait<0>();
+          drain();
           return;
         }
     ++passes;
@@ -612,7 +680,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
     if (dead || it == a.max_iters || (a.tol > 0.f && it == next_check)) {
       // the residual reads every contact: all updates of this sweep first
       if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) {
-        cp_wait<0>();
+        drain();
         return;
       }
       // Every scene has its own residual, summed in an order that neither the
@@ -645,7 +713,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
         }
       }
       if (!grid_barrier(d.bar, d.err, gen, d.wait_ns)) {
-        cp_wait<0>();
+        drain();
         return;
       }
       const uint32_t S = d.nscenes;
@@ -738,7 +806,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       done = s_flag || it == a.max_iters;
     }
   }
-  cp_wait<0>();
+  drain();
   if (blockIdx.x == 0) {
     // statistics: the sweeps done (the most any scene did), the largest final
     // residual, and per scene its sweeps x its contacts (the solver's work)
@@ -845,7 +913,7 @@ __global__ void __launch_bounds__(512) k_impact(DevPtrs d, ImpactArgs a) {
         const Row r = load_row(d, p);
         Side A, B;
         load_pair(d, r, A, B);
-        d.p_rq[p].y = r.qn + a.ups * (dot(r.n, B.v - A.v) - d.p_il2[p].z);
+        row_tile(d, p).rq[p & 31u].y = r.qn + a.ups * (dot(r.n, B.v - A.v) - d.p_il2[p].z);
       }
 }
 
@@ -859,7 +927,7 @@ __global__ void k_writeback(DevPtrs d) {
     if (c == 0xFFFFFFFFu) continue;  // padding slot
     float4 L0 = d.p_la[p];
     float2 L1 = d.p_lb[p];
-    float3 n = f3(d.p_rn[p]), t1, t2;
+    float3 n = f3(row_tile(d, p).rn[p & 31u]), t1, t2;
     onb(n, t1, t2);
     float3 tw = L0.y * t1 + L0.z * t2;
     d.prev_other[1][c] = (uint32_t)(d.c_key[c] & 0xFFFFFFFFull);
@@ -944,12 +1012,13 @@ __global__ void __launch_bounds__(256) k_tool(DevPtrs d, StepConsts k) {
   for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < first[ncol]; t += gridDim.x * blockDim.x) {
     while (t >= first[col + 1]) ++col;
     const uint32_t p = start[col] + (t - first[col]);
-    uint2 ab = d.p_ab[p];
+    const RowTile &row = row_tile(d, p);
+    const uint2 ab = row.ab[p & 31u];
     const uint32_t sid = d.sid[ab.x];
     const SceneGeo &G = k.geo[sid];
     if ((ab.y & ~TDS_STATIC) < 1u + G.nwall) continue;
-    float4 rn = d.p_rn[p], L0 = d.p_la[p];
-    float2 L1 = d.p_lb[p];
+    const float4 rn = row.rn[p & 31u], L0 = d.p_la[p];
+    const float2 L1 = d.p_lb[p];
     float3 n = f3(rn), t1, t2;
     onb(n, t1, t2);
     float3 F = (1.0f / k.dt) * (L0.x * n + L0.y * t1 + L0.z * t2);
