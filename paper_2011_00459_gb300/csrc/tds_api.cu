@@ -470,7 +470,7 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
 }
 
 int pgs_blocks_for(uint32_t n, int max_coop) {
-  int b = (int)((n + 127) / 128);
+  int b = (int)((n + 13) / 14);  // about a CTA per row tile (2 contacts a particle and more), up to the whole machine
   if (b < 1) b = 1;
   return b < max_coop ? b : max_coop;
 }
