@@ -321,6 +321,7 @@ __global__ void __launch_bounds__(TDS_NBUCKETS) k_bucket_starts(DevPtrs d) {
   for (uint32_t p = start + cnt; p < start + padded; ++p) {
     d.order[p] = 0xFFFFFFFFu;
     row_tile(d, p).ab[p & 31u] = make_uint2(~0u, ~0u);
+    row_tile(d, p).rk[p & 31u] = 0u;
   }
   if (b == 0u) {
     d.bstart[TDS_NBUCKETS] = total;

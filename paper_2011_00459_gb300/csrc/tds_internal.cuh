@@ -81,8 +81,8 @@ __device__ __forceinline__ int cell_axis(float x, float x0, float inv, int n) {
 // cell inside it (coordinates clamped to the block, which keeps neighbouring
 // particles in neighbouring cells). z runs fastest, then y, then x: beds are
 // wide and shallow, so slot order walks vertical columns slab by slab and a
-// particle's neighbours lie within about one x-slab of it in slot order (the
-// solver's CTAs then touch only nearby slot ranges).
+// particle's neighbours lie within about one x-slab of it in slot order (their
+// records then share L1 lines and L2 sectors).
 __device__ __forceinline__ uint32_t cell_index(const StepConsts &k, const SceneGeo &G, uint32_t sid, float4 p,
                                                int &cx, int &cy, int &cz) {
   cx = cell_axis(p.x, G.lo[0], k.cell_inv, k.gnx);
@@ -186,7 +186,7 @@ struct alignas(128) RowTile {
   float4 im[32];    // 1/m_a, 1/I_a, 1/m_b, 1/I_b (0 for a static side)
   uint2 ab[32];     // slot a, slot b | TDS_STATIC + surface id
   float2 rm[32];    // (mu, rbar mu_r)
-  uint32_t rk[32];  // rank and degree of the contact at a, then at b (a byte each)
+  uint32_t rk[32];  // rank and degree of the contact at a, then at b (a byte each); 0: not swept
 };
 __device__ __forceinline__ RowTile &row_tile(const DevPtrs &d, uint32_t p) {
   return reinterpret_cast<RowTile *>(d.p_rows)[p >> 5];

@@ -314,6 +314,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
 __device__ __forceinline__ void mbar_init(uint32_t bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void mbar_inval(uint32_t bar) {
+  asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -388,7 +391,7 @@ __device__ __forceinline__ Row settled_pair(const DevPtrs &d, uint32_t p, Side &
 // (rows staged by a TMA warp, every colour a barrier between neighbouring
 // CTAs), same box, ms for 100 sweeps: 1M spheres (3.2M contacts) 8.57 against
 // 12.1, 200k 2.55 against 5.76, 50k 1.61 against 3.34; 2000 spheres, 50 sweeps
-// 0.51 against 1.18; 64 beds of 406k spheres in all, 50 sweeps 1.34 against
+// 0.45 against 1.18; 64 beds of 406k spheres in all, 50 sweeps 1.34 against
 // 2.64.
 //  - 16 warps an SM with 128 registers each: 26 warps with 72 registers spill,
 //    and spilling took half of the L1 traffic (1M spheres 17.2 ms); 20 or 24
@@ -409,7 +412,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ double s_rn[kResSum], s_rd[kResSum];
   static_assert(kThreads >= (int)kResSum, "the residual sum needs kResSum threads");
-  __shared__ int s_flag;
+  __shared__ int s_flag, s_news;
   __shared__ uint32_t s_done[TDS_MAX_SCENES / 32], s_done_new[TDS_MAX_SCENES / 32];
   __shared__ uint32_t s_rmax, s_ndone, s_ndone_check, s_next;
   __shared__ unsigned long long s_acc[2];
@@ -456,21 +459,16 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
     total += __shfl_sync(0xffffffffu, incl, 31);
   }
   __syncwarp();
-  const uint32_t ntile = warp < total ? (total - warp + nwarps - 1u) / nwarps : 0u;
-  const uint2 *list = d.tiles + warp;
+  uint32_t ntile = warp < total ? (total - warp + nwarps - 1u) / nwarps : 0u;
+  uint2 *list = d.tiles + warp;
 
   // (the ring's tiles stay 128-byte aligned: the barriers come after all of them)
   const uint32_t ring = smem_u32(smem) + (threadIdx.x >> 5) * (uint32_t)(kRing * kTileBytes);
   unsigned char *ring_p = smem + (size_t)(threadIdx.x >> 5) * (kRing * kTileBytes);
   const uint32_t bars = smem_u32(smem) + (kThreads / 32) * (uint32_t)(kRing * kTileBytes) + (threadIdx.x >> 5) * (kRing * 8u);
-  if (lane == 0) {
-    for (int k = 0; k < kRing; ++k) mbar_init(bars + 8u * k);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncwarp();
   // lane l keeps entry l of the list's current group of 32
-  uint2 ent = lane < ntile ? list[(size_t)lane * nwarps] : make_uint2(0u, 0u);
-  uint32_t group = 0;
+  uint2 ent;
+  uint32_t group;
   auto entry = [&](uint32_t j) {
     if ((j >> 5) != group) {  // lists of more than 32 tiles
       group = j >> 5;
@@ -483,14 +481,14 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
   // The ring holds all of the warp's tiles: they are fetched once, and the
   // impulses live in it. Otherwise a tile is fetched again every sweep, at
   // least one tile after its impulses were stored.
-  const bool resident = ntile <= (uint32_t)kRing;
-  const uint32_t stages = resident ? ntile : (uint32_t)kRing;
+  bool resident;
+  uint32_t stages;
   bool dead = false;  // this warp's wait gave up (the error is latched)
   uint32_t it = 0;
-  uint32_t fetch = 0, fst = 0, st = 0;  // next tile to fetch, its ring stage, the current tile's stage
-  uint32_t fetched = 0, taken = 0;      // tiles fetched, and waited for, since the start
-  uint32_t tst = 0, tparity = 0;        // the next tile to wait for: its stage, its barrier's phase
-  uint32_t first_of[kAhead + 1];        // first contact of the current tile and the ones fetched after it
+  uint32_t fetch, fst, st;        // next tile to fetch, its ring stage, the current tile's stage
+  uint32_t fetched, taken;        // tiles fetched, and waited for, since the ring was started
+  uint32_t tst, tparity;          // the next tile to wait for: its stage, its barrier's phase
+  uint32_t first_of[kAhead + 1];  // first contact of the current tile and the ones fetched after it
   auto fetch_next = [&](bool on) {
     if (on) {
       const uint32_t p0 = entry(fetch).x, stage = ring + fst * (uint32_t)kTileBytes;
@@ -524,11 +522,6 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
     cp_wait<0>();
     while (taken < fetched) (void)take_rows(fetched);  // (a wait that runs out counts as taken)
   };
-#pragma unroll
-  for (int k = 0; k < kAhead; ++k) {
-    fetch_next(ntile > 0 && (!resident || k < (int)ntile));
-    first_of[k] = first_of[kAhead];
-  }
   // The records of a tile are read one tile ahead: whether they hold the
   // versions it needs is looked at when its turn comes, and only those that
   // did not are read again.
@@ -545,8 +538,27 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       nwb = __ldg(d.p_sw + p);
     }
   };
-  dead = !take_rows(1);
-  if (ntile > 0 && !dead) load_sides(ring_p, entry(0).x + lane);
+  // (Re)starts the ring at the list's first tile; no copy is in flight.
+  auto start_ring = [&] {
+    if (lane == 0) {
+      for (int k = 0; k < kRing; ++k) mbar_init(bars + 8u * k);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    resident = ntile <= (uint32_t)kRing;
+    stages = resident ? ntile : (uint32_t)kRing;
+    ent = lane < ntile ? list[(size_t)lane * nwarps] : make_uint2(0u, 0u);
+    group = 0;
+    fetch = fst = st = fetched = taken = tst = tparity = 0;
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) {
+      fetch_next(ntile > 0 && (!resident || k < (int)ntile));
+      first_of[k] = first_of[kAhead];
+    }
+    dead = !take_rows(1);
+    if (ntile > 0 && !dead) load_sides(ring_p, entry(0).x + lane);
+  };
+  start_ring();
 
   // residual checks: every `every` sweeps, or (every == 0) where the decay
   // seen so far says the tolerance will be met (see below)
@@ -557,7 +569,6 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
   bool done = a.max_iters == 0 && !warm;
   while (!done) {
     const bool warm_pass = passes < warm;
-    const bool skip_done = s_ndone != 0u;
     uint32_t col = 0;
     for (uint32_t j = 0; j < ntile && !dead; ++j) {
       if (!a.sync)  // grid barrier after every colour
@@ -566,7 +577,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
             drain();
             return;
           }
-      fetch_next(!resident || (passes == 0 && kAhead + j < ntile));
+      fetch_next(!resident || fetched < ntile);
       cp_wait<kAhead>();  // this tile's impulses are here
       dead = !take_rows(resident ? ntile : taken + 1u);  // and the next tile's rows
       if (dead) break;
@@ -580,8 +591,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       const float4 *s_rq = reinterpret_cast<const float4 *>(stage + kOffRq * 32) + lane;
       const float4 *s_im = reinterpret_cast<const float4 *>(stage + kOffIm * 32) + lane;
       const uint2 ab = reinterpret_cast<const uint2 *>(stage + kOffAb * 32)[lane];
-      bool live = ab.x != ~0u;
-      if (live && skip_done) live = !scene_done(s_done, __ldcg(d.sid + ab.x));
+      const uint32_t rk = reinterpret_cast<const uint32_t *>(stage + kOffRk * 32)[lane];
+      const bool live = rk != 0u;  // (0: padding, or a contact of a stopped scene)
       const bool dyn = is_dyn(ab.y);
       float4 *rec_a = d.rec + 2 * (size_t)ab.x, *rec_b = d.rec + 2 * (size_t)ab.y;
       float4 va = nva, wa = nwa, vb = nvb, wb = nwb;
@@ -593,7 +604,6 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       float2 L1;
       Pre pre;
       if (live) {
-        const uint32_t rk = reinterpret_cast<const uint32_t *>(stage + kOffRk * 32)[lane];
         want_a = passes * ((rk >> 8) & 0xFFu) + (rk & 0xFFu);
         want_b = passes * (rk >> 24) + ((rk >> 16) & 0xFFu);
         // computed while the records are on their way (the empty asm keeps it here)
@@ -789,6 +799,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       }
       __syncthreads();
       if (threadIdx.x == 0) {
+        s_news = s_ndone_check != s_ndone;
         s_ndone = s_ndone_check;
         // the largest residual of the scenes still sweeping (0 when all stopped)
         resid = __uint_as_float(s_rmax);
@@ -813,6 +824,47 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       __syncthreads();
       next_check = s_next;
       done = s_flag || it == a.max_iters;
+      if (s_news && !done) {
+        // Tiles whose scenes have all stopped leave the list, and a stopped
+        // scene's contacts in the tiles that stay lose their ranks (they then
+        // count as padding): the last sweeps of a batch cost what its
+        // unfinished beds cost. A tile's contacts are in owner order, so its
+        // scenes are the ones from its first contact's to its last one's; 32
+        // tiles at a time, a lane each.
+        // 256 beds to the 1e-4 residual (cap 2000 sweeps): 156 against 253 ms a step.
+        cp_wait<0>();
+        dead = !take_rows(fetched);
+        if (dead) continue;
+        uint32_t kept = 0;
+        for (uint32_t j0 = 0; j0 < ntile; j0 += 32u) {
+          uint2 e = make_uint2(0u, 0u);
+          bool keep = false, mixed = false;
+          if (j0 + lane < ntile) {
+            e = list[(size_t)(j0 + lane) * nwarps];
+            const uint2 *ab = row_tile(d, e.x).ab;
+            const uint32_t q1 = __ldcg(d.sid + __ldcg(ab + (e.y & 0xFFu) - 1u).x);
+            for (uint32_t q = __ldcg(d.sid + __ldcg(ab).x); q <= q1; ++q) {
+              const bool off = scene_done(s_done, q);
+              keep |= !off;
+              mixed |= off;
+            }
+          }
+          const uint32_t keeps = __ballot_sync(0xffffffffu, keep);
+          if (keep) list[(size_t)(kept + __popc(keeps & ((1u << lane) - 1u))) * nwarps] = e;
+          kept += __popc(keeps);
+          for (uint32_t m = __ballot_sync(0xffffffffu, keep && mixed); m; m &= m - 1u) {
+            RowTile &t = row_tile(d, __shfl_sync(0xffffffffu, e.x, __ffs(m) - 1));
+            const uint32_t i = __ldcg(t.ab + lane).x;
+            if (i != ~0u && scene_done(s_done, __ldcg(d.sid + i))) t.rk[lane] = 0u;
+          }
+        }
+        asm volatile("fence.proxy.async;" ::: "memory");  // the bulk copies read the ranks
+        __syncwarp();
+        ntile = kept;
+        if (lane == 0)
+          for (int k = 0; k < kRing; ++k) mbar_inval(bars + 8u * k);
+        start_ring();
+      }
     }
   }
   drain();
