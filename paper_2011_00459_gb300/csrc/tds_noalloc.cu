@@ -28,6 +28,7 @@
 #include <string>
 
 #include "tds_internal.cuh"
+#include "tds_rules.cuh"
 
 namespace {
 
@@ -134,18 +135,9 @@ __global__ void __launch_bounds__(256) k_plan(View v, const float *x, const floa
     __threadfence();
     for (int q = 0; q < 7; ++q) m[q] = unordered(*(volatile uint32_t *)(v.bounds() + q));
     for (int a = 0; a < 3; ++a) m[a] = -m[a];
-    float cell = 2.0f * m[6] * 1.025f * 1.02f;
-    if (!(cell > 0.f)) cell = 1.f;
+    const float extent[3] = {m[3] - m[0], m[4] - m[1], m[5] - m[2]};
     int dims[3];
-    for (;;) {
-      unsigned long long tot = 1;
-      for (int a = 0; a < 3; ++a) {
-        dims[a] = (int)ceilf((m[3 + a] - m[a]) / cell) + 1;
-        tot *= (unsigned long long)dims[a];
-      }
-      if (tot <= kMaxCells) break;
-      cell *= 1.25f;
-    }
+    const float cell = grid_plan(extent, 2.0f * m[6] * 1.025f * 1.02f, kMaxCells, dims);
     Plan *P = v.plan();
     for (int a = 0; a < 3; ++a) P->lo[a] = m[a];
     P->inv = 1.0f / cell;
