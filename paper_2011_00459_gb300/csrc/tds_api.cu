@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "tds_internal.cuh"
+#include "tds_rules.cuh"
 
 // launchers (tds_contacts.cu, tds_colour.cu, tds_solve.cu, tds_mlp.cu)
 int tds_launch_broadphase(const DevPtrs &d, const StepConsts &k, uint32_t ncells, cudaStream_t st);
@@ -316,22 +317,25 @@ Layout plan(const tds_scene_desc *descs, uint32_t S) {
   // cells wider than any reach (2 r_max plus the cohesive band), with margin
   L.cell = 2.0f * rmax * 1.025f * 1.02f;
   std::vector<float> lo(3 * S), hi(3 * S);
-  for (;;) {
+  constexpr uint32_t kMaxCells = 1u << 26;
+  for (;; L.cell = coarser(L.cell)) {  // coarser cells keep the grid bounded; correctness is unaffected
     int dims[3] = {1, 1, 1};
+    bool fits = true;
     for (uint32_t s = 0; s < S; ++s) {
       scene_domain(descs + s, L.cell, &lo[3 * s], &hi[3 * s]);
       for (int a = 0; a < 3; ++a) {
-        int n = (int)std::ceil((hi[3 * s + a] - lo[3 * s + a]) / L.cell);
-        dims[a] = std::max(dims[a], std::max(n, 1));
+        const int c = cells_along(hi[3 * s + a] - lo[3 * s + a], L.cell, kMaxCells);
+        fits &= c >= 0;
+        dims[a] = std::max(dims[a], c);
       }
     }
-    uint64_t tot = (uint64_t)S * dims[0] * dims[1] * dims[2];
-    if (tot <= (1ull << 26)) {
+    uint64_t tot = S;
+    for (int a = 0; a < 3 && tot <= kMaxCells; ++a) tot *= (uint64_t)dims[a];  // (each factor at most 2^26)
+    if (fits && tot <= kMaxCells) {
       L.gnx = dims[0]; L.gny = dims[1]; L.gnz = dims[2];
       L.ncells = (uint32_t)tot;
       break;
     }
-    L.cell *= 1.25f;  // coarser cells keep the grid bounded; correctness is unaffected
   }
   L.geo.resize(S);
   uint32_t hoff = 0, boff = 0, coff = 0, pid0 = 0;
