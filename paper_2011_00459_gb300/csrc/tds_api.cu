@@ -42,6 +42,7 @@ int tds_launch_cut(const DevPtrs &d, const StepConsts &k, float *heights, uint32
 void tds_launch_stage(const DevPtrs &d, uint32_t n, cudaStream_t st);
 int tds_pgs_setup();
 int tds_pgs_occupancy(int i);
+int tds_impact_occupancy();
 int tds_launch_aggregate(const DevPtrs &d, uint32_t n, const tds_zone *zones, uint32_t nz, uint8_t *zone_id,
                          double *sums, tds_aggregate *out, cudaStream_t st);
 size_t tds_aggregate_sums_words();
@@ -177,6 +178,7 @@ struct tds_scene {
   int pgs_blocks = 1, colour_blocks = 1;
   int pgs_sync = 1;       // solver: 1 waits per particle, 0 grid barrier between colours
   int pgs_shape = 0;      // solver CTA shape (index of the compiled shapes)
+  int max_impact_blocks = 1;  // co-resident CTAs of the impact stage
   bool any_cutter = false;
   int max_pgs_blocks = 1, max_colour_blocks = 1;
   int sms = 1;
@@ -675,15 +677,16 @@ tds_status create_impl(const tds_scene_desc *descs, uint32_t count, void *worksp
     if (descs[q].n_tool_boxes)
       h.tools.assign(descs[q].tool_boxes, descs[q].tool_boxes + 10 * descs[q].n_tool_boxes);
   }
-  int dev = 0, sms = 0, occ_pgs = 0, occ_col = 0;
+  int dev = 0, sms = 0, occ_pgs = 0, occ_imp = 0, occ_col = 0;
   cudaError_t ce = cudaGetDevice(&dev);
   if (ce == cudaSuccess) ce = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (ce == cudaSuccess) occ_pgs = tds_pgs_setup();
+  if (ce == cudaSuccess) occ_imp = tds_impact_occupancy();
   if (ce == cudaSuccess) ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_col, tds_colour_kernel(), 256, 0);
-  if (ce != cudaSuccess || occ_pgs < 1 || occ_col < 1) {
+  if (ce != cudaSuccess || occ_pgs < 1 || occ_imp < 1 || occ_col < 1) {
     delete s;
     if (ce == cudaSuccess)
-      return fail(TDS_ERR_CUDA, "a solver or colouring CTA shape does not fit on one SM (shared memory or "
+      return fail(TDS_ERR_CUDA, "a solver, impact or colouring CTA shape does not fit on one SM (shared memory or "
                                 "registers)");
     return fail(TDS_ERR_CUDA, std::string("device query failed: ") + cudaGetErrorString(ce));
   }
@@ -694,6 +697,7 @@ tds_status create_impl(const tds_scene_desc *descs, uint32_t count, void *worksp
   // the rounds' barriers
   s->colour_blocks = std::max(1, (int)std::min<uint64_t>((uint64_t)sms * (occ_col < 4 ? occ_col : 4),
                                                          ((uint64_t)s->L.n * 4 + 255) / 256));
+  s->max_impact_blocks = sms * occ_imp;
   s->max_pgs_blocks = 64 * sms;  // the workspace's limit; each shape's co-residency limits it further
   s->max_colour_blocks = sms * occ_col;
   Carver probe{nullptr};
@@ -857,7 +861,9 @@ tds_status enqueue_step(tds_scene *s, cudaEvent_t *E, uint64_t &launches, bool c
   }
   launches += tds_launch_bucketing(d, s->L.cap, s->st);
   if (D.impact_iters > 0) {
-    CUDA_TRY(tds_launch_impact(d, s->k, D.restitution, D.impact_speed, D.impact_iters, s->pgs_blocks, s->st));
+    // the solver's CTAs, as far as the stage's own fit (its loops take any number)
+    CUDA_TRY(tds_launch_impact(d, s->k, D.restitution, D.impact_speed, D.impact_iters,
+                               std::min(s->pgs_blocks, s->max_impact_blocks), s->st));
     launches += 1 + tds_launch_records(d, s->L.n, s->st);
   }
   if (E) CUDA_TRY(cudaEventRecordWithFlags(E[3], s->st, evf));

@@ -920,7 +920,8 @@ struct ImpactArgs {
   uint32_t iters;
 };
 
-__global__ void __launch_bounds__(512) k_impact(DevPtrs d, ImpactArgs a) {
+constexpr int kImpactThreads = 512;
+__global__ void __launch_bounds__(kImpactThreads) k_impact(DevPtrs d, ImpactArgs a) {
   if (step_failed(d)) return;
   __shared__ uint32_t s_count;
   const uint32_t ncol = min(d.ctr[CTR_NCOL], (uint32_t)TDS_MAX_COLOURS);
@@ -1194,7 +1195,7 @@ cudaError_t tds_launch_impact(const DevPtrs &d, const StepConsts &k, float e, fl
   cudaMemsetAsync(d.ctr + CTR_IMPACTS, 0, sizeof(uint32_t), st);
   DevPtrs dd = d;
   void *args[] = {&dd, &a};
-  return cudaLaunchCooperativeKernel((const void *)k_impact, dim3(blocks), dim3(512), args, 0, st);
+  return cudaLaunchCooperativeKernel((const void *)k_impact, dim3(blocks), dim3(kImpactThreads), args, 0, st);
 }
 
 // Opt the solver into its shared-memory stages; returns the co-resident
@@ -1218,6 +1219,12 @@ int tds_pgs_setup() {
 
 // Co-resident CTAs per SM of compiled shape i (after tds_pgs_setup).
 int tds_pgs_occupancy(int i) { return g_pgs_occupancy[i]; }
+
+// Co-resident CTAs per SM of the impact stage (0: none, or the query failed).
+int tds_impact_occupancy() {
+  int occ = 0;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void *)k_impact, kImpactThreads, 0) == cudaSuccess ? occ : 0;
+}
 
 int tds_launch_finish(const DevPtrs &d, const StepConsts &k, uint32_t cap, cudaStream_t st) {
   k_writeback<<<grid_for(cap, 256), 256, 0, st>>>(d);
