@@ -43,3 +43,17 @@ TDS_HD float grid_plan(const float extent[3], float cell, uint32_t max_cells, in
     if (fits && total <= max_cells) return cell;
   }
 }
+
+// The check word of a solver record, four 64-bit words that each move whole:
+// (v.x, v.y), (v.z, version), (w.x, w.y), (w.z, check). The second carries its
+// version itself; check ties the other three to it: the version and what the
+// first and third hold, each word rotated by its own amount, so that changes
+// of several words by the same bits (equal components, a version and a
+// velocity that both change in their last bit) do not cancel, as they would
+// in a plain exclusive or. (The amounts differ by no multiple of 8: the
+// rotations of equal words by 0, 8, 16 and 24 cancel for one word in 256.)
+TDS_HD uint32_t rotl(uint32_t x, int r) { return (x << r) | (x >> (32 - r)); }
+TDS_HD uint32_t check_of_version(uint32_t version) { return rotl(version, 22) ^ 0x5bd1e995u; }
+TDS_HD uint32_t record_check(uint32_t of_version, uint32_t vx, uint32_t vy, uint32_t wx, uint32_t wy) {
+  return of_version ^ vx ^ rotl(vy, 5) ^ rotl(wx, 10) ^ rotl(wy, 15);
+}
