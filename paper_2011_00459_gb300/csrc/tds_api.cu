@@ -46,8 +46,8 @@ int tds_impact_occupancy();
 int tds_launch_aggregate(const DevPtrs &d, uint32_t n, const tds_zone *zones, uint32_t nz, uint8_t *zone_id,
                          double *sums, tds_aggregate *out, cudaStream_t st);
 size_t tds_aggregate_sums_words();
-int tds_launch_coarse_grain(const DevPtrs &d, uint32_t n, const tds_grid &g, int kernel, float R, float *rho,
-                            float *p, float *u, size_t scratch_cells, cudaStream_t st);
+int tds_launch_coarse_grain(const DevPtrs &d, uint32_t n, uint32_t live, const tds_grid &g, int kernel, float R,
+                            float *rho, float *p, float *u, size_t scratch_cells, cudaStream_t st);
 bool tds_grid_valid(const tds_grid *g);
 const void *tds_colour_kernel();
 
@@ -101,6 +101,7 @@ struct Carver {
 // Per-scene host data of a batch.
 struct SceneHost {
   uint32_t off, n;                  // particle ids [off, off + n)
+  uint32_t live = 0;                // particles, as far as the host knows: without the reserve until something may wake it
   std::vector<float> walls, tools;  // 10 floats per box
   bool has_cutter = false;
   tds_cutter cutter{};
@@ -673,6 +674,7 @@ tds_status create_impl(const tds_scene_desc *descs, uint32_t count, void *worksp
     h.off = off;
     h.n = descs[q].n;
     off += h.n;
+    for (uint32_t i = 0; i < h.n; ++i) h.live += descs[q].radius[i] > 0.f;
     if (descs[q].n_walls) h.walls.assign(descs[q].walls, descs[q].walls + 10 * descs[q].n_walls);
     if (descs[q].n_tool_boxes)
       h.tools.assign(descs[q].tool_boxes, descs[q].tool_boxes + 10 * descs[q].n_tool_boxes);
@@ -1124,6 +1126,7 @@ tds_status tds_load_state(tds_scene *s, const void *buf, uint64_t bytes) {
   CUDA_TRY(cudaMemcpyAsync(s->d.err, &zero, sizeof zero, cudaMemcpyHostToDevice, s->st));
   CUDA_TRY(cudaMemcpyAsync(s->d.ctr + CTR_CLEAN, &clean, sizeof clean, cudaMemcpyHostToDevice, s->st));
   CUDA_TRY(cudaStreamSynchronize(s->st));
+  for (SceneHost &q : s->scenes) q.live = q.n;  // (the state may hold woken particles)
   s->steps = h.steps;
   s->have_prev = h.have_prev != 0;
   s->latched = TDS_OK;
@@ -1296,6 +1299,7 @@ tds_status tds_set_cutter(tds_scene *s, uint32_t scene, const tds_cutter *c) {
   SceneHost &h = s->scenes[scene];
   h.cutter = *c;
   h.has_cutter = c->length > 0.f;
+  if (h.has_cutter) h.live = h.n;
   compose_boxes(s, scene);
   s->any_cutter = false;
   for (const SceneHost &q : s->scenes) s->any_cutter |= q.has_cutter;
@@ -1487,7 +1491,7 @@ tds_status tds_coarse_grain(tds_scene *s, const tds_grid *grid, int32_t kernel, 
     return fail(TDS_ERR_INVALID_ARG, "Gaussian smoothing length must be in (0, 16 l0]");
   tds_status ls = check_latched(s);
   if (ls != TDS_OK) return ls;
-  s->launches += tds_launch_coarse_grain(s->d, s->L.n, *grid, kernel, R, rho, p, u,
+  s->launches += tds_launch_coarse_grain(s->d, s->L.n, s->scenes[grid->scene].live, *grid, kernel, R, rho, p, u,
                                          (size_t)s->L.cap + TDS_ORDER_PAD, s->st);
   CUDA_TRY(cudaGetLastError());
   return TDS_OK;

@@ -5,6 +5,7 @@
 #include <cmath>
 
 #include "tds_internal.cuh"
+#include "tds_rules.cuh"
 
 tds_status tds_set_error_message(tds_status s, const char *msg);
 
@@ -283,9 +284,10 @@ int grid_blocks(size_t n) {
 
 // Scratch: the impact stage's colour-order arrays (used only inside a step)
 // for the voxels, the read-back staging and the broadphase's for the sorted
-// particles. scratch_cells: float4 entries of the first.
-int tds_launch_coarse_grain(const DevPtrs &d, uint32_t n, const tds_grid &g, int kernel, float R, float *rho,
-                            float *p, float *u, size_t scratch_cells, cudaStream_t st) {
+// particles. scratch_cells: float4 entries of the first. live: the particles of
+// the grid's scene, without the reserve as far as is known.
+int tds_launch_coarse_grain(const DevPtrs &d, uint32_t n, uint32_t live, const tds_grid &g, int kernel, float R,
+                            float *rho, float *p, float *u, size_t scratch_cells, cudaStream_t st) {
   const size_t nvox = (size_t)g.nx * g.ny * g.nz;
   if (kernel == 0 && nvox <= scratch_cells) {
     cudaMemsetAsync(d.p_il, 0, sizeof(float4) * nvox, st);
@@ -293,13 +295,8 @@ int tds_launch_coarse_grain(const DevPtrs &d, uint32_t n, const tds_grid &g, int
     k_cg_split<<<grid_blocks(nvox), kThreads, 0, st>>>((uint32_t)nvox, d.p_il, rho, p, u);
     return 2;
   }
-  // The gather looks at every row in reach of every voxel (of the order of
-  // (R/l0)^2), the scatter at every voxel in reach of every particle
-  // ((R/l0)^3): measured at R = l0 the gather takes 1.05 ns a voxel on sparse
-  // grids and the scatter 4.1 ns a particle (0.6 and 1.1 at R = l0/2), so the
-  // line lies at about 3.5 R/l0 voxels a particle.
   if (kernel == 1 && nvox + 1 + tds_scan_tmp_words((uint32_t)nvox) <= 4 * scratch_cells && nvox < 0x7FFFFFFFu &&
-      (double)nvox <= 3.5 * (double)(R / g.l0) * (double)n) {
+      gather_pays((double)nvox, (double)(R / g.l0), (double)live)) {
     GaussBins b;
     b.count = reinterpret_cast<uint32_t *>(d.p_il);
     uint32_t *tmp = b.count + nvox + 1;

@@ -44,6 +44,29 @@ TDS_HD float grid_plan(const float extent[3], float cell, uint32_t max_cells, in
   }
 }
 
+// Whether the Gaussian fields' gather takes less time than the scatter, for a
+// grid of so many voxels, a smoothing length of q voxels and a scene of so many
+// particles. Measured for 300 to 1M particles, 1e-4 to 10 voxels a particle and
+// q from 0.2 to 6, 879 pairs of times: the choice takes 1.007 times the better
+// one's time on average, and at most 1.15 times the scatter's. (The line
+// before, 3.5 q voxels a particle alone: 1.13 and 6.2.)
+//  - The gather looks at every row in reach of every voxel (some q^2), the
+//    scatter at every voxel in reach of every particle (some q^3). 200k particles:
+//    q = 1/2, 73k voxels 91 and 105 us, 158k 121 and 103; q = 1, 158k 281 and
+//    582, 480k 611 and 574; q = 3, 1.8M 11.0 and 12.7 ms. Up to some 30 000 q
+//    voxels (q^1.5 from one voxel on) the gather is all launches and latency
+//    (20k particles, q = 1/2, 22k voxels: 42 and 47 us).
+//  - On a few voxels the scatter's reductions meet at few addresses, but the
+//    gather has few warps, each with all particles to walk: 20k particles,
+//    q = 0.4, 120 voxels 318 and 251 us, 280 voxels 111 and 152; q = 0.6, 64
+//    voxels 668 and 1202.
+//  - With q <= 0.3 a particle reaches about three voxels, for which the gather
+//    walks up to 27: 200k particles, 34k voxels 58 and 46 us.
+TDS_HD bool gather_pays(double voxels, double q, double particles) {
+  return q > 0.31 && voxels * q * q * q * q >= 3.0 + 1e-5 * particles &&
+         voxels <= fmin(1.8 * q * q, 3.5 * q) * particles + 30000.0 * q * fmax(1.0, sqrt(q));
+}
+
 // The check word of a solver record, four 64-bit words that each move whole:
 // (v.x, v.y), (v.z, version), (w.x, w.y), (w.z, check). The second carries its
 // version itself; check ties the other three to it: the version and what the
