@@ -46,7 +46,7 @@ int tds_impact_occupancy();
 int tds_launch_aggregate(const DevPtrs &d, uint32_t n, const tds_zone *zones, uint32_t nz, uint8_t *zone_id,
                          double *sums, tds_aggregate *out, cudaStream_t st);
 size_t tds_aggregate_sums_words();
-int tds_launch_coarse_grain(const DevPtrs &d, uint32_t n, uint32_t live, const tds_grid &g, int kernel, float R,
+int tds_launch_coarse_grain(const DevPtrs &d, uint32_t n, double live, const tds_grid &g, int kernel, float R,
                             float *rho, float *p, float *u, size_t scratch_cells, cudaStream_t st);
 bool tds_grid_valid(const tds_grid *g);
 const void *tds_colour_kernel();
@@ -102,6 +102,7 @@ struct Carver {
 struct SceneHost {
   uint32_t off, n;                  // particle ids [off, off + n)
   uint32_t live = 0;                // particles, as far as the host knows: without the reserve until something may wake it
+  double volume = 0.0;              // of a particle, on average at creation (0: none yet)
   std::vector<float> walls, tools;  // 10 floats per box
   bool has_cutter = false;
   tds_cutter cutter{};
@@ -674,7 +675,12 @@ tds_status create_impl(const tds_scene_desc *descs, uint32_t count, void *worksp
     h.off = off;
     h.n = descs[q].n;
     off += h.n;
-    for (uint32_t i = 0; i < h.n; ++i) h.live += descs[q].radius[i] > 0.f;
+    for (uint32_t i = 0; i < h.n; ++i) {
+      const double r = descs[q].radius[i];
+      h.live += r > 0.0;
+      h.volume += 4.0 / 3.0 * M_PI * r * r * r;
+    }
+    if (h.live) h.volume /= h.live;
     if (descs[q].n_walls) h.walls.assign(descs[q].walls, descs[q].walls + 10 * descs[q].n_walls);
     if (descs[q].n_tool_boxes)
       h.tools.assign(descs[q].tool_boxes, descs[q].tool_boxes + 10 * descs[q].n_tool_boxes);
@@ -1491,7 +1497,14 @@ tds_status tds_coarse_grain(tds_scene *s, const tds_grid *grid, int32_t kernel, 
     return fail(TDS_ERR_INVALID_ARG, "Gaussian smoothing length must be in (0, 16 l0]");
   tds_status ls = check_latched(s);
   if (ls != TDS_OK) return ls;
-  s->launches += tds_launch_coarse_grain(s->d, s->L.n, s->scenes[grid->scene].live, *grid, kernel, R, rho, p, u,
+  // the particles that can lie within the kernel's reach of the grid: all of the
+  // scene's, or as many as a packed bed (0.64) has there
+  const SceneHost &h = s->scenes[grid->scene];
+  double live = h.live;
+  if (h.volume > 0.0)
+    live = std::fmin(live, 0.64 / h.volume * (grid->nx * (double)grid->l0 + 6.0 * R) *
+                               (grid->ny * (double)grid->l0 + 6.0 * R) * (grid->nz * (double)grid->l0 + 6.0 * R));
+  s->launches += tds_launch_coarse_grain(s->d, s->L.n, live, *grid, kernel, R, rho, p, u,
                                          (size_t)s->L.cap + TDS_ORDER_PAD, s->st);
   CUDA_TRY(cudaGetLastError());
   return TDS_OK;
