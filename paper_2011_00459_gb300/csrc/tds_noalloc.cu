@@ -271,8 +271,8 @@ struct WideRow {  // the row of the lowest lane in m, known to all lanes
 };
 
 template <bool kWrite, bool kCrowded>
-__device__ __forceinline__ void pairs(View v, uint32_t n, unsigned long long *keys, uint32_t cap, uint32_t *count_out) {
-  const Plan P = *v.plan();
+__device__ __forceinline__ void pairs(View v, const Plan P, uint32_t n, unsigned long long *keys, uint32_t cap,
+                                      uint32_t *count_out) {
   const float4 *sp = v.spos();
   const uint32_t *sid = v.sid();
   if (kWrite && blockIdx.x == 0 && threadIdx.x == 0) *count_out = v.cstart()[n];
@@ -342,8 +342,9 @@ __device__ __forceinline__ void pairs(View v, uint32_t n, unsigned long long *ke
 template <bool kWrite>
 __global__ void __launch_bounds__(128, 16) k_pairs(View v, uint32_t n, unsigned long long *keys, uint32_t cap,
                                                    uint32_t *count_out) {
-  if (*v.nbig() == 0u) pairs<kWrite, false>(v, n, keys, cap, count_out);
-  else pairs<kWrite, true>(v, n, keys, cap, count_out);
+  const Plan P = *v.plan();
+  if (*v.nbig() == 0u) pairs<kWrite, false>(v, P, n, keys, cap, count_out);
+  else pairs<kWrite, true>(v, P, n, keys, cap, count_out);
 }
 
 std::mutex g_mu;
