@@ -401,9 +401,10 @@ __device__ __forceinline__ Row settled_pair(const DevPtrs &d, uint32_t p, Side &
 // 12.1, 200k 2.55 against 5.76, 50k 1.61 against 3.34; 2000 spheres, 50 sweeps
 // 0.45 against 1.18; 64 beds of 406k spheres in all, 50 sweeps 1.34 against
 // 2.64.
-//  - 16 warps an SM with 128 registers each: 26 warps with 72 registers spill,
-//    and spilling took half of the L1 traffic (1M spheres 17.2 ms); 20 or 24
-//    warps that do not read records ahead 8.99 and 9.92 against 8.77.
+//  - 16 warps an SM with 128 registers each, which read records ahead (8.63
+//    ms): with 20, 24 and 26 warps (640x2, 768x1, 416x1) there are no registers
+//    for it, 8.9, 10.2 and 11.7. On the batch of 64 beds 640x2 is 1 % faster
+//    (1.346 against 1.364), on 2000 spheres 14 % slower.
 //  - Tiles in turn rather than a stretch of slots per warp: every warp gets the
 //    same number (2000 spheres 0.70 against 1.48 ms), and dependent tiles are
 //    a whole colour apart.
@@ -416,6 +417,12 @@ template <int kThreads, int kPerThread, int kMinBlocks>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveArgs a) {
   constexpr int kRing = ring_tiles(kPerThread);  // tiles in a warp's ring
   constexpr int kAhead = kRing - 1;              // tiles fetched ahead
+  // Shapes of up to 16 warps an SM read the next tile's records ahead and work
+  // this one's rows out during the wait. The others have too few registers for
+  // it: with both they spilled 750 bytes a thread (416x1) and took 19.9 ms (1M
+  // spheres, 100 sweeps; 768x1 and 256x1 16.0, 640x2 13.1); without, 200 bytes
+  // and 11.7 ms (10.2, 10.2 and 8.9).
+  constexpr bool kReadAhead = kThreads * kMinBlocks <= 512;
   if (step_failed(d)) return;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ double s_rn[kResSum], s_rd[kResSum];
@@ -564,7 +571,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       first_of[k] = first_of[kAhead];
     }
     dead = !take_rows(1);
-    if (ntile > 0 && !dead) load_sides(ring_p, entry(0).x + lane);
+    if (kReadAhead && ntile > 0 && !dead) load_sides(ring_p, entry(0).x + lane);
   };
   start_ring();
 
@@ -603,8 +610,12 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
       const bool live = rk != 0u;  // (0: padding, or a contact of a stopped scene)
       const bool dyn = is_dyn(ab.y);
       float4 *rec_a = d.rec + 2 * (size_t)ab.x, *rec_b = d.rec + 2 * (size_t)ab.y;
+      if (!kReadAhead) {
+        nva = nwa = nvb = nwb = make_float4(0.f, 0.f, 0.f, 0.f);  // (nothing is carried over)
+        load_sides(stage, p);
+      }
       float4 va = nva, wa = nwa, vb = nvb, wb = nwb;
-      if (ntile > 1) load_sides(ring_p + st * kTileBytes, p_next);
+      if (kReadAhead && ntile > 1) load_sides(ring_p + st * kTileBytes, p_next);
       uint32_t want_a = 0, want_b = 0, chk_a = 0, chk_b = 0;  // versions, and their parts of the check words
       bool need_a = live, need_b = live && dyn;
       Row r;
@@ -617,7 +628,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
         chk_a = check_of_version(want_a);
         chk_b = check_of_version(want_b);
         asm volatile("" : "+r"(chk_a), "+r"(chk_b));  // (here, not after the wait)
-        // computed while the records are on their way (the empty asm keeps it here)
+      }
+      auto read_row = [&] {
         const float4 rn = *s_rn, rq = *s_rq;
         im = *s_im;
         r.n = f3(rn); r.la = rn.w;
@@ -629,6 +641,10 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
         Side A, B;
         A.im = im.x; A.iI = im.y; B.im = im.z; B.iI = im.w;
         pre = prepare_update(r, A, B, a.sig_t, a.sig_r);
+      };
+      if (kReadAhead && live) {
+        // computed while the records are on their way (the empty asm keeps it here)
+        read_row();
         asm volatile("" : "+f"(pre.iDn), "+f"(pre.iDt), "+f"(pre.iDr), "+f"(pre.t1.x), "+f"(pre.t1.y), "+f"(pre.t1.z),
                      "+f"(pre.t2.x), "+f"(pre.t2.y), "+f"(pre.t2.z)::"memory");
       }
@@ -671,6 +687,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
         }
       }
       if (live && !dead) {
+        if (!kReadAhead) read_row();
         float4 &s_la = reinterpret_cast<float4 *>(stage + kOffLa * 32)[lane];
         float2 &s_lb = reinterpret_cast<float2 *>(stage + kOffLb * 32)[lane];
         Side A{f3(va), f3(wa), im.x, im.y}, B{f3(vb), f3(wb), im.z, im.w};
@@ -691,7 +708,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
           }
         }
       }
-      if (ntile == 1) load_sides(stage, p);
+      if (kReadAhead && ntile == 1) load_sides(stage, p);
     }
     if (!a.sync)
       for (; col < ncol; ++col)
