@@ -7,9 +7,10 @@ persistent solver's CTA count and its synchronisation between colours
 Every setting gives bit-identical results, so the tuner only picks the
 fastest: it times a few steps of the caller's own scene (continuing its
 motion) per candidate with CUDA events on the scene's stream and keeps the
-best. Choices are cached as JSON per GPU model and workload shape (particles
-rounded to two significant digits, and scenes), so a later run with the same
-shape reuses them without timing.
+best. Choices are cached as JSON per GPU model, workload shape (particles
+rounded to two significant digits, scenes, impact stage) and schedule (the
+solver's version and its compiled shapes), so a later run with the same shape
+reuses them without timing, and one with another solver times its own.
 """
 from __future__ import annotations
 
@@ -37,8 +38,8 @@ def _round2(x: float) -> int:
     return int(round(x / 10 ** e) * 10 ** e)
 
 
-def shape_key(gpu: str, particles: int, scenes: int) -> str:
-    return f"{gpu}|n={_round2(particles)}|scenes={scenes}"
+def shape_key(gpu: str, particles: int, scenes: int, impact: bool = False) -> str:
+    return f"{gpu}|n={_round2(particles)}|scenes={scenes}|impact={int(impact)}|{schedule()}"
 
 
 def load_cache(path: str | None = None) -> dict:
@@ -67,6 +68,16 @@ def store_cache(key: str, entry: dict, path: str | None = None) -> None:
 SYNC_MODES = (1, 0)  # per particle, grid barrier
 # solver CTA shapes the library compiles: (threads, row tiles in flight per warp, CTAs per SM)
 SHAPES = ((512, 2, 1), (416, 1, 2), (768, 1, 1), (640, 2, 1), (512, 3, 1), (256, 1, 3))
+# Counted up whenever the solver's schedule changes (what a shape's numbers mean, which is fast): a choice timed on
+# another schedule is not used. 1: rows staged by a TMA warp, barriers between colours; 2: versioned records, row tiles;
+# 3: without records read ahead in shapes of more than 16 warps an SM.
+SCHEDULE = 3
+
+
+def schedule() -> str:
+    return f"schedule={SCHEDULE}:" + ",".join(f"{t}x{per}x{k}" for t, per, k in SHAPES)
+
+
 KEYS = ("pgs_blocks", "pgs_sync", "colour_blocks", "pgs_threads", "pgs_per_thread")
 
 
@@ -129,7 +140,7 @@ def tune(sim, steps: int = 3, sweeps: int = 50, use_cache: bool = True, path: st
     g = sim.g
     cfg = g.launch_config()
     props = torch.cuda.get_device_properties(torch.cuda.current_device())
-    key = shape_key(props.name, g.n, len(g.sizes))
+    key = shape_key(props.name, g.n, len(g.sizes), g.impact)
     if use_cache:
         hit = load_cache(path).get(key)
         if hit and all(k in hit.get("shape", {}) for k in KEYS):

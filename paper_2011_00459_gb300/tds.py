@@ -318,6 +318,7 @@ class Scene:
         self.n = int(self.offsets[-1])
         self.desc = descs[0]
         self.solver = (int(descs[0].max_iters), float(descs[0].tol), int(descs[0].residual_every))
+        self.impact = descs[0].impact_iters > 0  # the impact stage is on
         self._descs = descs
         self._keep = keep
         L = lib()
@@ -414,6 +415,7 @@ class Scene:
     def set_impact(self, restitution: float, impact_speed: float, iters: int):
         """Impact stage settings (iters 0 disables it)."""
         _check(lib().tds_set_impact(self.h, float(restitution), float(impact_speed), int(iters)))
+        self.impact = int(iters) > 0
 
     def set_cutter(self, cutter: dict | None, scene: int = 0):
         """Active-zone cutter on the scene's tool (tool-frame edge point,
