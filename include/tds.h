@@ -443,6 +443,9 @@ tds_status tds_load_state(tds_scene *s, const void *buf, uint64_t bytes);
  * contact rows each of its warps keeps in flight, one of the compiled shapes
  * 512x2 (the default), 768x1, 640x2, 512x3 (one CTA per SM), 416x1 (two CTAs
  * per SM) and 256x1 (three CTAs per SM) (both 0 keep the current shape).
+ * More pgs_blocks than a chosen shape's co-resident CTAs are refused; while
+ * no shape has been chosen, up to two per SM are taken (an earlier default
+ * shape held as many) and lowered to what fits.
  * max_pgs_blocks / max_colour_blocks (read only) are the co-resident limits
  * (max_pgs_blocks for the current solver shape; a shape change with
  * pgs_blocks 0 lowers the solver CTAs to the new shape's limit if needed).

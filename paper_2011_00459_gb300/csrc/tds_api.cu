@@ -180,6 +180,7 @@ struct tds_scene {
   int pgs_blocks = 1, colour_blocks = 1;
   int pgs_sync = 1;       // solver: 1 waits per particle, 0 grid barrier between colours
   int pgs_shape = 0;      // solver CTA shape (index of the compiled shapes)
+  bool own_shape = false; // the caller has chosen it
   int max_impact_blocks = 1;  // co-resident CTAs of the impact stage
   bool any_cutter = false;
   int max_pgs_blocks = 1, max_colour_blocks = 1;
@@ -1213,17 +1214,20 @@ tds_status tds_set_launch_config(tds_scene *s, const tds_launch_config *cfg) {
     }
   }
   // the solver CTAs must all be co-resident: at most the SMs times the
-  // chosen shape's CTAs per SM
+  // chosen shape's CTAs per SM. A caller that never chose a shape may ask for up
+  // to two per SM, as many as an earlier default shape had, and gets what fits.
   const int max_blocks = std::min(64 * s->sms, s->sms * tds_pgs_occupancy(shape));
-  if (cfg->pgs_blocks > max_blocks)
+  const bool own = s->own_shape || cfg->pgs_threads;
+  if (cfg->pgs_blocks > (own ? max_blocks : std::max(max_blocks, 2 * s->sms)))
     return fail(TDS_ERR_INVALID_ARG, "pgs_blocks exceeds the co-resident CTAs of that solver shape (" +
                                          std::to_string(max_blocks) + ")");
-  if (cfg->pgs_blocks) s->pgs_blocks = cfg->pgs_blocks;
+  if (cfg->pgs_blocks) s->pgs_blocks = std::min(cfg->pgs_blocks, max_blocks);
   else if (s->pgs_blocks > max_blocks) s->pgs_blocks = max_blocks;
   if (cfg->colour_blocks) s->colour_blocks = cfg->colour_blocks;
   if (cfg->wait_limit_us) s->d.wait_ns = 1000ull * (unsigned long long)cfg->wait_limit_us;
   s->pgs_sync = cfg->pgs_sync;
   s->pgs_shape = shape;
+  s->own_shape = own;
   return TDS_OK;
 }
 

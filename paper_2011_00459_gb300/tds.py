@@ -522,8 +522,7 @@ class Scene:
         c.wait_limit_us = int(wait_limit_us)
         if pgs_sync is not None:
             c.pgs_sync = int(pgs_sync)
-        if pgs_threads or pgs_per_thread:
-            c.pgs_threads, c.pgs_per_thread = int(pgs_threads), int(pgs_per_thread)
+        c.pgs_threads, c.pgs_per_thread = int(pgs_threads), int(pgs_per_thread)  # (both 0: the current shape)
         _check(lib().tds_set_launch_config(self.h, ctypes.byref(c)))
 
     def set_graph(self, enable: bool = True):
