@@ -9,6 +9,7 @@
 // particles, 8 zones: 39 and 44 us; with FP64 divisions, conversions and five
 // shuffle steps and additions per component and 32 particles 146 and 185.
 // k_agg_final 6.4 us against 24.
+#include <cfloat>
 #include <cstring>
 
 #include "tds_internal.cuh"
@@ -56,10 +57,14 @@ __device__ __forceinline__ double widen(float x) {
 // Mass of a particle: the reciprocal of the FP32 record's 1/m. FP64 division
 // costs about twenty FP64 operations, which this GPU issues at a sixty-fourth
 // of the FP32 rate; Newton's iteration r <- r + r (1 - a r) doubles the correct
-// digits of the FP32 reciprocal, to 2^-46 and then to the last bit.
+// digits of the FP32 reciprocal, to 2^-46 and then to the last bit. Where that
+// reciprocal is no normal number (masses beyond FP32's range, an infinite or a
+// zero one) the iteration has nothing to start from, and the division is taken.
 __device__ __forceinline__ double mass_of(float inv_m) {
   const double a = widen(inv_m);
-  double r = widen(__frcp_rn(inv_m));
+  const float start = __frcp_rn(inv_m);
+  if (!(start >= FLT_MIN && start <= FLT_MAX)) return 1.0 / a;
+  double r = widen(start);
   r = fma(r, fma(-a, r, 1.0), r);
   return fma(r, fma(-a, r, 1.0), r);
 }
