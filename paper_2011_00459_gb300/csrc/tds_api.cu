@@ -39,7 +39,7 @@ cudaError_t tds_launch_impact(const DevPtrs &d, const StepConsts &k, float e, fl
                               int blocks, cudaStream_t st);
 int tds_launch_finish(const DevPtrs &d, const StepConsts &k, uint32_t cap, cudaStream_t st);
 int tds_launch_cut(const DevPtrs &d, const StepConsts &k, float *heights, uint32_t nh, cudaStream_t st);
-void tds_launch_stage(const DevPtrs &d, uint32_t n, cudaStream_t st);
+void tds_launch_stage(const DevPtrs &d, uint32_t n, bool id_order, cudaStream_t st);
 int tds_pgs_setup();
 int tds_pgs_occupancy(int i);
 int tds_impact_occupancy();
@@ -174,6 +174,7 @@ struct tds_scene {
   void *mem = nullptr;
   bool owns = false;
   bool have_prev = false;
+  bool id_order = true;   // the slots are in id order still: neither stepped nor loaded
   std::vector<SceneHost> scenes;
   std::vector<BoxF> host_boxes;
   bool geo_dirty = true;
@@ -978,7 +979,7 @@ tds_status read_particles_impl(tds_scene *s, uint32_t off, uint32_t count, float
                                float *vx, float *vy, float *vz, float *wx, float *wy, float *wz) {
   tds_status ls = check_latched(s);
   if (ls != TDS_OK) return ls;
-  tds_launch_stage(s->d, s->L.n, s->st);
+  tds_launch_stage(s->d, s->L.n, s->id_order, s->st);
   float *outs[9] = {x, y, z, vx, vy, vz, wx, wy, wz};
   for (int q = 0; q < 9; ++q)
     if (outs[q])
@@ -1134,6 +1135,7 @@ tds_status tds_load_state(tds_scene *s, const void *buf, uint64_t bytes) {
   CUDA_TRY(cudaMemcpyAsync(s->d.ctr + CTR_CLEAN, &clean, sizeof clean, cudaMemcpyHostToDevice, s->st));
   CUDA_TRY(cudaStreamSynchronize(s->st));
   for (SceneHost &q : s->scenes) q.live = q.n;  // (the state may hold woken particles)
+  s->id_order = false;
   s->steps = h.steps;
   s->have_prev = h.have_prev != 0;
   s->latched = TDS_OK;
@@ -1267,6 +1269,7 @@ tds_status tds_step(tds_scene *s, uint32_t nsteps) {
     if (r != TDS_OK) return r;
     s->parity ^= 1u;
     s->have_prev = true;
+    s->id_order = false;
     s->steps++;
   }
   CUDA_TRY(cudaGetLastError());
@@ -1338,7 +1341,7 @@ tds_status tds_read_radii(tds_scene *s, float *r, uint32_t n) {
   if (n != s->L.n) return fail(TDS_ERR_INVALID_ARG, "n differs from the particle count");
   tds_status ls = check_latched(s);
   if (ls != TDS_OK) return ls;
-  tds_launch_stage(s->d, s->L.n, s->st);
+  tds_launch_stage(s->d, s->L.n, s->id_order, s->st);
   CUDA_TRY(cudaMemcpyAsync(r, s->d.stage + (size_t)9 * s->L.n, sizeof(float) * n, cudaMemcpyDeviceToHost, s->st));
   return sync_and_check(s);
 }

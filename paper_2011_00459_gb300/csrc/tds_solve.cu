@@ -1152,7 +1152,10 @@ __global__ void __launch_bounds__(256) k_tool(DevPtrs d, StepConsts k) {
 // beds first each id's slot and then the records gathered by id: whole sectors
 // read and coalesced writes (1M particles 27 us in two launches against 72 of
 // ten scattered 4-byte writes a particle); up to kStageScatter particles one
-// launch that scatters is as fast (2000: 4 us against 6).
+// launch that scatters (whole calls on settled beds, scattered and gathered:
+// 32k particles 56 and 58 us, 65k 64 and 66, 131k 87 and 80, 262k 112 and 109,
+// 1M 280 and 268). A scene that has not been stepped has its slots in id order:
+// the scatter's writes are coalesced, and it is one launch (1M: 243 and 253).
 constexpr uint32_t kStageScatter = 65536;
 
 __global__ void k_slots(DevPtrs d, uint32_t n) {
@@ -1261,8 +1264,8 @@ int tds_launch_finish(const DevPtrs &d, const StepConsts &k, uint32_t cap, cudaS
   return 3;
 }
 
-void tds_launch_stage(const DevPtrs &d, uint32_t n, cudaStream_t st) {
-  if (n <= kStageScatter) {
+void tds_launch_stage(const DevPtrs &d, uint32_t n, bool id_order, cudaStream_t st) {
+  if (id_order || n <= kStageScatter) {
     k_stage<false><<<grid_for(n, 256), 256, 0, st>>>(d, n);
     return;
   }
