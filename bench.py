@@ -19,6 +19,8 @@ as separate scenes.
             roofline is the persistent PGS kernel's algorithmic bytes (204 B
             per particle-pair contact and 160 B per static contact per sweep)
             over its CUDA-event time there, against the measured HBM copy peak
+            (frac); records and part of the rows come from L2, so what the HBM
+            itself does is dram_frac, the captured DRAM bytes over that time
   cpu_baseline: the FP64 CPU oracle on a bounded column of the same bed
 
 ``--impl reference`` times the oracle alone (the slow baseline arm).
@@ -183,11 +185,11 @@ def measured_peaks() -> dict:
 
 
 def pgs_source_sha() -> str:
-    """Hash of the solver's code (tds_solve.cu and tds_internal.cuh with
-    comments and blank lines removed): the ncu counters stay valid while it
-    is unchanged."""
+    """Hash of the solver's code (tds_solve.cu, tds_internal.cuh and
+    tds_rules.cuh with comments and blank lines removed): the ncu counters
+    stay valid while it is unchanged."""
     h = hashlib.sha256()
-    for f in ("tds_solve.cu", "tds_internal.cuh"):
+    for f in ("tds_solve.cu", "tds_internal.cuh", "tds_rules.cuh"):
         src = open(os.path.join(ROOT, "paper_2011_00459_gb300", "csrc", f)).read()
         src = re.sub(r"/\*.*?\*/", "", src, flags=re.S)
         src = re.sub(r"//[^\n]*", "", src)
@@ -978,6 +980,9 @@ def main():
     per = ncu_traffic(args.workload)
     sweeps_contacts = rst["sweep_contacts_pp"] + rst["sweep_contacts_static"]
     traffic = per * sweeps_contacts / max(1, rst["solved_steps"]) if per is not None else None
+    # what crosses HBM: the captured bytes over the same time (records and part of the rows come from L2, so the
+    # algorithmic rate above can exceed the HBM peak)
+    dram = traffic * max(1, rst["solved_steps"]) / (pgs_ms * 1e-3) / 1e9 if traffic is not None and pgs_ms > 0 else None
     phase = lambda q: {k: v / max(1, q["timed_steps"]) for k, v in q["phase_ms"].items()}
     result = {
         "metric": METRIC, "value": n_all * args.steps / (ms * 1e-3), "unit": UNIT,
@@ -993,6 +998,7 @@ def main():
                    "phase_ms_per_step": phase(st)},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                      "frac": achieved / peaks["hbm_gbs"], "traffic": traffic,
+                     "dram_gbs": dram, "dram_frac": dram / peaks["hbm_gbs"] if dram is not None else None,
                      "kernel": "k_pgs (persistent colour-sweep PGS)",
                      "region": (f"second timed region: {fixed['sweeps']} fixed sweeps per step, {args.steps} "
                                 f"steps of the same bed continuing its dig" if fixed else "the headline region"),

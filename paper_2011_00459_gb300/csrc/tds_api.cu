@@ -184,7 +184,7 @@ struct tds_scene {
   bool own_shape = false; // the caller has chosen it
   int max_impact_blocks = 1;  // co-resident CTAs of the impact stage
   bool any_cutter = false;
-  int max_pgs_blocks = 1, max_colour_blocks = 1;
+  int max_colour_blocks = 1;
   int sms = 1;
   uint64_t steps = 0;
   tds_status latched = TDS_OK;
@@ -382,7 +382,7 @@ Layout plan(const tds_scene_desc *descs, uint32_t S) {
   return L;
 }
 
-size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
+size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x) {
   const uint32_t n = L.n, cap = L.cap;
   d.pos = c.take<float4>(n); d.pv = c.take<float4>(2 * (size_t)n);
   d.rec = c.take<float4>(2 * (size_t)n);
@@ -431,9 +431,7 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x, int pgs_blocks) {
   d.ctr = c.take<uint32_t>(CTR_COUNT);
   d.acc = c.take<unsigned long long>(ACC_COUNT);
   d.fscal = c.take<float>(FS_COUNT);
-  size_t nd = 2 * (size_t)pgs_blocks;
-  if (nd < 6 * 128) nd = 6 * 128;
-  d.dpart = c.take<double>(nd);
+  d.dpart = c.take<double>(6 * TDS_TOOL_BLOCKS);
   const size_t nsb = (size_t)L.S * TDS_NBUCKETS;
   const size_t max_chunks = (size_t)cap / TDS_RES_CHUNK + nsb + 1;
   d.dres = c.take<double>(2 * max_chunks);
@@ -652,9 +650,7 @@ tds_status workspace_bytes_impl(const tds_scene_desc *descs, uint32_t count, uin
   DevPtrs d{};
   Extra x;
   Carver c{nullptr};
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  *bytes = carve(c, L, d, x, 64 * sms);
+  *bytes = carve(c, L, d, x);
   return TDS_OK;
 }
 
@@ -708,12 +704,11 @@ tds_status create_impl(const tds_scene_desc *descs, uint32_t count, void *worksp
   s->colour_blocks = std::max(1, (int)std::min<uint64_t>((uint64_t)sms * (occ_col < 4 ? occ_col : 4),
                                                          ((uint64_t)s->L.n * 4 + 255) / 256));
   s->max_impact_blocks = sms * occ_imp;
-  s->max_pgs_blocks = 64 * sms;  // the workspace's limit; each shape's co-residency limits it further
   s->max_colour_blocks = sms * occ_col;
   Carver probe{nullptr};
   DevPtrs tmp{};
   Extra tx;
-  size_t need = carve(probe, s->L, tmp, tx, 64 * sms);
+  size_t need = carve(probe, s->L, tmp, tx);
   if (workspace) {
     if (workspace_bytes < need) {
       delete s;
@@ -729,7 +724,7 @@ tds_status create_impl(const tds_scene_desc *descs, uint32_t count, void *worksp
     s->owns = true;
   }
   Carver c{(char *)s->mem};
-  carve(c, s->L, s->d, s->x, 64 * sms);
+  carve(c, s->L, s->d, s->x);
   s->d.targ = nullptr;
   s->d.wait_ns = TDS_BARRIER_NS;
   s->d.recolour = 1u;
@@ -1181,7 +1176,7 @@ tds_status tds_get_launch_config(tds_scene *s, tds_launch_config *out) {
   out->pgs_blocks = s->pgs_blocks;
   out->pgs_sync = s->pgs_sync;
   out->colour_blocks = s->colour_blocks;
-  out->max_pgs_blocks = std::min(s->max_pgs_blocks, s->sms * tds_pgs_occupancy(s->pgs_shape));
+  out->max_pgs_blocks = s->sms * tds_pgs_occupancy(s->pgs_shape);
   out->max_colour_blocks = s->max_colour_blocks;
   tds_pgs_shape(s->pgs_shape, &out->pgs_threads, &out->pgs_per_thread);
   out->wait_limit_us = (int32_t)(s->d.wait_ns / 1000ull);
@@ -1218,7 +1213,7 @@ tds_status tds_set_launch_config(tds_scene *s, const tds_launch_config *cfg) {
   // the solver CTAs must all be co-resident: at most the SMs times the
   // chosen shape's CTAs per SM. A caller that never chose a shape may ask for up
   // to two per SM, as many as an earlier default shape had, and gets what fits.
-  const int max_blocks = std::min(64 * s->sms, s->sms * tds_pgs_occupancy(shape));
+  const int max_blocks = s->sms * tds_pgs_occupancy(shape);
   const bool own = s->own_shape || cfg->pgs_threads;
   if (cfg->pgs_blocks > (own ? max_blocks : std::max(max_blocks, 2 * s->sms)))
     return fail(TDS_ERR_INVALID_ARG, "pgs_blocks exceeds the co-resident CTAs of that solver shape (" +

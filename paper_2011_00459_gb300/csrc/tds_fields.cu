@@ -161,13 +161,6 @@ __global__ void __launch_bounds__(kThreads) k_cg_place(DevPtrs d, uint32_t n, fl
 
 constexpr int kMaxRows = 101;  // rows of voxels across the reach along one axis (R <= 16 l0)
 
-// A warp per voxel; its four groups of eight lanes take the rows in turn (runs
-// of voxels along x, whose particles are contiguous) that can hold a particle
-// within 3R, a lane per particle. The rows are taken longest first, so that
-// the four in work at a time have about the same length. A row is cut to the
-// voxels in reach: the particles of a voxel da rows away are at least
-// (|da| - 1/2) l0 from the centre along that axis (those of a border voxel,
-// which also holds what lies outside the grid, even more).
 // 2^x by the hardware's approximation (relative error at most 2^-22, as
 // expf's). The argument r2 (-log2 e / 2 R^2) is two roundings from the exact
 // one, expf's -r2 (1 / 2 R^2) three; expf's own arithmetic was a quarter of the
@@ -178,6 +171,13 @@ __device__ __forceinline__ float exp2_approx(float x) {
   return y;
 }
 
+// A warp per voxel; its four groups of eight lanes take the rows in turn (runs
+// of voxels along x, whose particles are contiguous) that can hold a particle
+// within 3R, a lane per particle. The rows are taken longest first, so that
+// the four in work at a time have about the same length. A row is cut to the
+// voxels in reach: the particles of a voxel da rows away are at least
+// (|da| - 1/2) l0 from the centre along that axis (those of a border voxel,
+// which also holds what lies outside the grid, even more).
 constexpr int kGatherBlocks = 6;  // per SM
 __global__ void __launch_bounds__(kThreads, kGatherBlocks) k_cg_gather(tds_grid g, float R, float exponent, int reach,
                                                                        GaussBins b, uint32_t nvox, float *rho,

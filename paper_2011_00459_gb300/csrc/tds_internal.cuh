@@ -12,6 +12,7 @@
 #define TDS_NBUCKETS (2 * TDS_MAX_COLOURS)  // (colour, static?) buckets
 #define TDS_TILE 2048                       // contacts per bucketing tile
 #define TDS_ORDER_PAD (32 * TDS_NBUCKETS)     // padding slots of the colour order
+#define TDS_TOOL_BLOCKS 64                   // blocks that add up the tool's force
 #define TDS_RES_CHUNK 256u                  // contacts per residual chunk (at most)
 #define TDS_BARRIER_NS 2000000000ull        // default limit of a wait on other CTAs (2 s); also the
                                             // fixed limit of a CTA's wait for its own bulk copies
@@ -156,7 +157,8 @@ struct DevPtrs {
   uint32_t *bar;              // grid barrier: [0] arrivals, [1] generation
   uint2 *tiles;               // solver: the warps' row tiles (first contact, contacts | bucket << 8)
   uint32_t *scan_tmp;
-  float *stage;               // 9 n floats for reads
+  float *stage;               // 10 n floats: read-back staging; scratch of the aggregate bodies (masses, 2 n) and
+                              // of the Gaussian fields (sorted particles, 10 n) between steps
   float *tool_out;            // 6 floats per scene
   double *tool_acc;           // per-scene force and torque accumulators (batches)
   // learned warm start (owner order)

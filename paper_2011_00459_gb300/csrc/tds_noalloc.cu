@@ -244,13 +244,13 @@ __global__ void __launch_bounds__(1024) k_cell_sort_big(View v, const float *x, 
 // a chain of loads: 20 us to count and 27 to write at 40 000 particles, against
 // 12.7 and 17.4.
 // Where there are cells of more than kSmallCell particles (coarsened by a far
-// particle or one large radius), rows of more than kLaneRow candidates are taken
-// by the whole warp, 32 candidates at a time, one row after another: with all
-// particles in one cell a lane's row holds all of them and the other eight none.
-// 40 001 particles and an outlier, the whole call: 7.1 ms, by lanes alone 31.6,
-// by a thread a particle 11.3; an outlier along one axis, 10 km away: 1.3, 4.4
-// and 3.6. (At 128 candidates the 27 rows
-// of a warp take about as many turns either way.)
+// particle or one large radius), rows of more than kLaneRow candidates are
+// taken by the whole warp, 32 candidates at a time, one row after another: with
+// all particles in one cell a lane's row holds all of them and the other eight
+// none. 40 001 particles and an outlier, the whole call: 7.1 ms, by lanes alone
+// 31.6, by a thread a particle 11.3; an outlier along one axis, 10 km away: 1.3,
+// 4.4 and 3.6. (At 128 candidates the 27 rows of a warp take about as many turns
+// either way.)
 constexpr uint32_t kLaneRow = 128;
 
 struct WideRow {  // the row of the lowest lane in m, known to all lanes

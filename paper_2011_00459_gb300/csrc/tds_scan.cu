@@ -4,7 +4,9 @@
 // (launches bound it there: one instead of three, 3.9 us against 9.4 for 2001
 // elements), more in two phases, tile sums and then a per-tile scan whose block
 // adds up the tiles before its own itself (a separate scan of the tile sums is
-// a launch and a pass of one block: 2.4 to 4 us more).
+// a launch and a pass of one block: 2.4 to 4 us more). Those sums are quadratic
+// in the tiles, from L2: with the largest grid (2^26 cells, 32768 tiles) 2 GB,
+// and still a step of 2000 spheres in it takes 0.75 ms against 1.48.
 #include "tds_internal.cuh"
 
 namespace {

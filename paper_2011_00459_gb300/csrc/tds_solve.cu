@@ -216,7 +216,6 @@ struct SolveArgs {
   float tol, sig_t, sig_r;
   int apply_warm;
   int sync;  // between colours: 0 grid barrier, 1 the particle records' versions alone
-  uint32_t n;  // particle slots
 };
 
 // ---------------------------------------------------------------------------
@@ -1058,10 +1057,10 @@ __global__ void k_integrate(DevPtrs d, StepConsts k, uint32_t cap) {
 // Soil-on-tool force and torque about the tool origin: sum over tool
 // contacts of (Lambda_n n + Lambda_t) / dt at the contact point, plus the
 // rolling impulse / dt. Only the static buckets hold tool contacts (all
-// contacts: 98 us on the 1M bed). Fixed block partition + fixed-order
-// sums, the blocks' added by the last one to finish: the result is
-// reproducible.
-constexpr int kToolBlocks = 64;
+// contacts: 98 us on the 1M bed). A single scene's result is reproducible:
+// fixed block partition and fixed-order sums, the blocks' added by the last one
+// to finish. A batch's scenes are added by FP64 atomics in any order, which the
+// rounding to FP32 hides but for ties.
 
 // Sums of six values per thread over a block of 256 threads, in threads 0 to 5.
 __device__ __forceinline__ double block_sum6(const double (&v)[6], double (*sh)[6]) {
@@ -1137,7 +1136,7 @@ __global__ void __launch_bounds__(256) k_tool(DevPtrs d, StepConsts k) {
   if (threadIdx.x == 0) d.ctr[CTR_TICKET] = 0u;  // for the next step
   if (k.nscenes == 1) {
 #pragma unroll
-    for (int q = 0; q < 6; ++q) acc[q] = threadIdx.x < kToolBlocks ? __ldcg(d.dpart + 6 * threadIdx.x + q) : 0.0;
+    for (int q = 0; q < 6; ++q) acc[q] = threadIdx.x < TDS_TOOL_BLOCKS ? __ldcg(d.dpart + 6 * threadIdx.x + q) : 0.0;
     const double s = block_sum6(acc, sh);
     if (threadIdx.x < 6) d.tool_out[threadIdx.x] = (float)s;
     return;
@@ -1210,7 +1209,7 @@ void tds_pgs_shape(int i, int *threads, int *per_thread) {
 
 cudaError_t tds_launch_pgs(const DevPtrs &d, const StepConsts &k, uint32_t max_iters, float tol,
                            uint32_t every, int apply_warm, int blocks, int sync, int shape, cudaStream_t st) {
-  SolveArgs a{max_iters, every, tol, k.sig_t, k.sig_r, apply_warm, sync, k.n};
+  SolveArgs a{max_iters, every, tol, k.sig_t, k.sig_r, apply_warm, sync};
   cudaMemsetAsync(d.bar, 0, 2 * sizeof(uint32_t), st);
   DevPtrs dd = d;
   void *args[] = {&dd, &a};
@@ -1259,7 +1258,7 @@ int tds_impact_occupancy() {
 
 int tds_launch_finish(const DevPtrs &d, const StepConsts &k, uint32_t cap, cudaStream_t st) {
   k_writeback<<<grid_for(cap, 256), 256, 0, st>>>(d);
-  k_tool<<<kToolBlocks, 256, 0, st>>>(d, k);
+  k_tool<<<TDS_TOOL_BLOCKS, 256, 0, st>>>(d, k);
   k_integrate<<<grid_for(k.n, 256), 256, 0, st>>>(d, k, cap);
   return 3;
 }
