@@ -442,7 +442,8 @@ tds_status tds_load_state(tds_scene *s, const void *buf, uint64_t bytes);
  * pgs_threads x pgs_per_thread: the solver CTA's threads and the tiles of 32
  * contact rows each of its warps keeps in flight, one of the compiled shapes
  * 512x2 (the default), 768x1, 640x2, 512x3 (one CTA per SM), 416x1 (two CTAs
- * per SM) and 256x1 (three CTAs per SM) (both 0 keep the current shape).
+ * per SM) and 256x1 (three CTAs per SM) (both 0 keep the current shape);
+ * a CTA of a bed with fewer row tiles than warps is launched with fewer.
  * More pgs_blocks than a chosen shape's co-resident CTAs are refused; while
  * no shape has been chosen, up to two per SM are taken (an earlier default
  * shape held as many) and lowered to what fits.

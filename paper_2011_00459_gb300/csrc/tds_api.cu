@@ -866,9 +866,11 @@ tds_status enqueue_step(tds_scene *s, cudaEvent_t *E, uint64_t &launches, bool c
   }
   launches += tds_launch_bucketing(d, s->L.cap, s->st);
   if (D.impact_iters > 0) {
-    // the solver's CTAs, as far as the stage's own fit (its loops take any number)
+    // the solver's CTAs, as far as the stage's own fit (its loops take any
+    // number), and no more than a thread per contact or so
+    const uint64_t enough = ((uint64_t)s->L.n * 4 + 511) / 512;
     CUDA_TRY(tds_launch_impact(d, s->k, D.restitution, D.impact_speed, D.impact_iters,
-                               std::min(s->pgs_blocks, s->max_impact_blocks), s->st));
+                               (int)std::min<uint64_t>(std::min(s->pgs_blocks, s->max_impact_blocks), enough), s->st));
     launches += 1 + tds_launch_records(d, s->L.n, s->st);
   }
   if (E) CUDA_TRY(cudaEventRecordWithFlags(E[3], s->st, evf));

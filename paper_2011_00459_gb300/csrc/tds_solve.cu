@@ -297,7 +297,7 @@ constexpr int kShapes[][3] = {{512, 2, 1}, {416, 1, 2}, {768, 1, 1}, {640, 2, 1}
 constexpr int kNumShapes = 6;
 constexpr int kStages = 1;                           // ring stages per row tile in flight (and one in use)
 constexpr uint32_t kFirstCheck = 5;                  // first residual check in adaptive mode
-constexpr uint32_t kResSum = 256;                    // residual: threads adding up a large scene's chunks
+constexpr uint32_t kResSum = 256;                    // residual: partial sums of a large scene's chunks
 constexpr uint32_t kWarpChunks = 1024;               // residual: scenes with at most this many chunks
                                                      // are added by one warp, larger ones by the CTA
 // A warp's ring holds row tiles (see RowTile) with their impulses. Per contact:
@@ -425,14 +425,14 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
   if (step_failed(d)) return;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ double s_rn[kResSum], s_rd[kResSum];
-  static_assert(kThreads >= (int)kResSum, "the residual sum needs kResSum threads");
   __shared__ int s_flag, s_news;
   __shared__ uint32_t s_done[TDS_MAX_SCENES / 32], s_done_new[TDS_MAX_SCENES / 32];
   __shared__ uint32_t s_rmax, s_ndone, s_ndone_check, s_next;
   __shared__ unsigned long long s_acc[2];
   const uint32_t ncol = min(d.ctr[CTR_NCOL], (uint32_t)TDS_MAX_COLOURS);
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t nwarps = gridDim.x * (kThreads / 32);
+  const uint32_t cta_warps = blockDim.x >> 5;  // kThreads / 32, or fewer for small beds (solver_warps)
+  const uint32_t nwarps = gridDim.x * cta_warps;
   if (threadIdx.x == 0) {
     s_ndone = 0;
     s_acc[0] = s_acc[1] = 0ull;
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
   // 2.91). With more, they lie on one SM and a tile finds its neighbours'
   // rows in the same part of DRAM and L2 (1M spheres 8.57 against 9.13 ms).
   const uint32_t warp = all <= 2u * nwarps ? (threadIdx.x >> 5) * gridDim.x + blockIdx.x
-                                           : blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+                                           : blockIdx.x * cta_warps + (threadIdx.x >> 5);
   uint32_t total = 0;
   for (uint32_t g0 = 0; g0 < 2 * ncol; g0 += 32) {
     const uint32_t g = g0 + lane;
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
   // (the ring's tiles stay 128-byte aligned: the barriers come after all of them)
   const uint32_t ring = smem_u32(smem) + (threadIdx.x >> 5) * (uint32_t)(kRing * kTileBytes);
   unsigned char *ring_p = smem + (size_t)(threadIdx.x >> 5) * (kRing * kTileBytes);
-  const uint32_t bars = smem_u32(smem) + (kThreads / 32) * (uint32_t)(kRing * kTileBytes) + (threadIdx.x >> 5) * (kRing * 8u);
+  const uint32_t bars = smem_u32(smem) + cta_warps * (uint32_t)(kRing * kTileBytes) + (threadIdx.x >> 5) * (kRing * 8u);
   // lane l keeps entry l of the list's current group of 32
   uint2 ent;
   uint32_t group;
@@ -771,9 +771,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
         const uint32_t c0 = __ldcg(d.scq_chunk + (size_t)q * TDS_NBUCKETS);
         const uint32_t c1 = __ldcg(d.scq_chunk + (size_t)(q + 1) * TDS_NBUCKETS);
         if (c1 - c0 <= kWarpChunks || scene_done(s_done, q)) continue;
-        if (threadIdx.x < kResSum) {
+        for (uint32_t t = threadIdx.x; t < kResSum; t += blockDim.x) {
           double n0 = 0.0, n1 = 0.0, d0 = 0.0, d1 = 0.0;
-          uint32_t ch = c0 + threadIdx.x;
+          uint32_t ch = c0 + t;
           for (; ch + kResSum < c1; ch += 2u * kResSum) {
             const double2 u = __ldcg(reinterpret_cast<const double2 *>(d.dres) + ch);
             const double2 v = __ldcg(reinterpret_cast<const double2 *>(d.dres) + ch + kResSum);
@@ -784,14 +784,14 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_pgs(DevPtrs d, SolveAr
             const double2 u = __ldcg(reinterpret_cast<const double2 *>(d.dres) + ch);
             n0 += u.x; d0 += u.y;
           }
-          s_rn[threadIdx.x] = n0 + n1;
-          s_rd[threadIdx.x] = d0 + d1;
+          s_rn[t] = n0 + n1;
+          s_rd[t] = d0 + d1;
         }
         __syncthreads();
         for (uint32_t h = kResSum / 2u; h > 0u; h >>= 1) {
-          if (threadIdx.x < h) {
-            s_rn[threadIdx.x] += s_rn[threadIdx.x + h];
-            s_rd[threadIdx.x] += s_rd[threadIdx.x + h];
+          for (uint32_t t = threadIdx.x; t < h; t += blockDim.x) {
+            s_rn[t] += s_rn[t + h];
+            s_rd[t] += s_rd[t + h];
           }
           __syncthreads();
         }
@@ -1213,7 +1213,7 @@ cudaError_t tds_launch_pgs(const DevPtrs &d, const StepConsts &k, uint32_t max_i
   cudaMemsetAsync(d.bar, 0, 2 * sizeof(uint32_t), st);
   DevPtrs dd = d;
   void *args[] = {&dd, &a};
-  const int T = kShapes[shape][0];
+  const int T = 32 * solver_warps(k.n, blocks, kShapes[shape][0] / 32);
   return cudaLaunchCooperativeKernel((const void *)kPgsKernels[shape], dim3(blocks), dim3(T), args,
                                      pgs_smem(T, kShapes[shape][1]), st);
 }
