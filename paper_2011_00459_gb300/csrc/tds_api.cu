@@ -402,12 +402,8 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x) {
   d.c_sv = c.take<float4>(cap); d.c_sw = c.take<float4>(cap);
   d.c_la = c.take<float4>(cap); d.c_lb = c.take<float2>(cap);
   d.inc_cnt = c.take<uint32_t>(n + 1); d.inc_start = c.take<uint32_t>(n + 1);
-  d.inc_ent = c.take<uint2>(2 * (size_t)cap);
-  d.prio = c.take<unsigned long long>(cap);
   d.colour = c.take<uint8_t>(cap);
   d.cmask = c.take<ulonglong2>(n);
-  d.wait = c.take<int32_t>(cap);
-  d.frontier0 = c.take<uint32_t>(cap); d.frontier1 = c.take<uint32_t>(cap);
   d.ntiles = L.ntiles;
   d.tile_hist = c.take<uint32_t>((size_t)TDS_NBUCKETS * L.ntiles);
   d.tile_off = c.take<uint32_t>((size_t)TDS_NBUCKETS * L.ntiles + 1);
@@ -416,7 +412,14 @@ size_t carve(Carver &c, const Layout &L, DevPtrs &d, Extra &x) {
   d.bpad = c.take<uint32_t>(TDS_NBUCKETS);
   const size_t pc = (size_t)cap + TDS_ORDER_PAD;  // colour order with padding
   d.order = c.take<uint32_t>(pc);
+  // the row tiles are written once the colouring is done, so its arrays lie in
+  // them: 36 bytes a contact in 68 (the padding's tiles exceed the alignments)
   d.p_rows = c.take<unsigned char>((pc / 32 + 1) * sizeof(RowTile));
+  Carver in{reinterpret_cast<char *>(d.p_rows)};
+  d.inc_ent = in.take<uint2>(2 * (size_t)cap);
+  d.prio = in.take<unsigned long long>(cap);
+  d.wait = in.take<int32_t>(cap);
+  d.frontier0 = in.take<uint32_t>(cap); d.frontier1 = in.take<uint32_t>(cap);
   d.p_sv = c.take<float4>(pc); d.p_sw = c.take<float4>(pc);
   d.p_la = c.take<float4>(pc); d.p_lb = c.take<float2>(pc);
   d.p_il = c.take<float4>(pc); d.p_il2 = c.take<float4>(pc);

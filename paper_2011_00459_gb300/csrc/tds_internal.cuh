@@ -115,7 +115,7 @@ struct DevPtrs {
   float4 *c_sv, *c_sw;        // static side: point velocity, spin
   float4 *c_la;               // initial impulses (n, t1, t2, r.x)
   float2 *c_lb;               // (r.y, r.z)
-  // colouring
+  // colouring (incidences, priorities, wait and frontiers lie where the row tiles are written afterwards)
   uint32_t *inc_cnt, *inc_start;
   uint2 *inc_ent;             // (contact id, high word of its priority) per incidence
   unsigned long long *prio;   // colouring priority per contact
