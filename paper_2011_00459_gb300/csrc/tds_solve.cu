@@ -396,10 +396,10 @@ __device__ __forceinline__ Row settled_pair(const DevPtrs &d, uint32_t p, Side &
 // the L1 data pipe (a record is one wavefront per lane and access), L2 and the
 // rows' DRAM traffic about equally. Measured against the solver this replaced
 // (rows staged by a TMA warp, every colour a barrier between neighbouring
-// CTAs), same box, ms for 100 sweeps: 1M spheres (3.2M contacts) 8.57 against
-// 12.1, 200k 2.55 against 5.76, 50k 1.61 against 3.34; 2000 spheres, 50 sweeps
-// 0.45 against 1.18; 64 beds of 406k spheres in all, 50 sweeps 1.34 against
-// 2.64.
+// CTAs), same box, ms for 100 sweeps: 1M spheres (3.2M contacts) 8.64 against
+// 12.1, 200k 2.55 against 5.05, 50k 1.59 against 3.45; 2000 spheres, 50 sweeps
+// 0.44 against 1.29; 64 beds of 406k spheres in all, 50 sweeps 1.35 against
+// 2.36.
 //  - 16 warps an SM with 128 registers each, which read records ahead (8.63
 //    ms): with 20, 24 and 26 warps (640x2, 768x1, 416x1) there are no registers
 //    for it, 8.9, 10.2 and 11.7. On the batch of 64 beds 640x2 is 1 % faster
