@@ -49,9 +49,13 @@ TDS_HD float grid_plan(const float extent[3], float cell, uint32_t max_cells, in
 // shape's. A warp beyond the tiles would only hold registers, which several
 // small scenes on their own streams can share: a round of steps of 16 scenes of
 // 2000 spheres, 50 sweeps, takes 1.95 ms, with 16 warps in every CTA 7.98; of 8000
-// spheres 5.9 and 10.3; one scene's step is as fast either way.
-TDS_HD int solver_warps(uint32_t n, int blocks, int most) {
-  const uint32_t want = (n / 8u + 64u + (uint32_t)blocks - 1u) / (uint32_t)blocks;
+// spheres 5.9 and 10.3; one scene's step is as fast either way. In a batch every
+// CTA also adds up every scene's residual, a warp each, so there also a warp for
+// eight scenes (1000 beds of 4 spheres, 100 sweeps, a check each: 56 ms, with one
+// warp 75).
+TDS_HD int solver_warps(uint32_t n, uint32_t scenes, int blocks, int most) {
+  const uint32_t tiles = (n / 8u + 64u + (uint32_t)blocks - 1u) / (uint32_t)blocks;
+  const uint32_t want = (scenes + 7u) / 8u > tiles ? (scenes + 7u) / 8u : tiles;
   return want < (uint32_t)most ? (int)want : most;
 }
 

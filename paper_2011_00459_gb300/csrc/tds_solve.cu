@@ -1213,7 +1213,7 @@ cudaError_t tds_launch_pgs(const DevPtrs &d, const StepConsts &k, uint32_t max_i
   cudaMemsetAsync(d.bar, 0, 2 * sizeof(uint32_t), st);
   DevPtrs dd = d;
   void *args[] = {&dd, &a};
-  const int T = 32 * solver_warps(k.n, blocks, kShapes[shape][0] / 32);
+  const int T = 32 * solver_warps(k.n, k.nscenes, blocks, kShapes[shape][0] / 32);
   return cudaLaunchCooperativeKernel((const void *)kPgsKernels[shape], dim3(blocks), dim3(T), args,
                                      pgs_smem(T, kShapes[shape][1]), st);
 }
